@@ -55,6 +55,14 @@ bool is_device_ptr(const void* p) {
 }
 
 constexpr long long kTimeoutCycles = 4000000000ll;  // about two seconds at 2 GHz per wait
+constexpr int kTeamBatchCluster = 8;               // cluster of a batch's teams
+constexpr long long kTeamCtaWork = 8192;           // a team has a CTA per so much work (nnz + 4 n)
+constexpr long long kTeamGridWork = 160 * 1000;    // from here a single system takes the whole grid
+constexpr size_t kTeamIndexHeap = 112 * 1024;      // shared memory up to which a team's columns are copied
+constexpr int kTeamIcRows = 32768;                 // IC(0) in a team: rows of the vector in shared memory
+constexpr size_t kTeamIcRing = 96 * 1024;          // ... bytes of its ring of level blocks at most
+constexpr size_t kTeamIcShared = 180 * 1024;       // ... and of both together
+constexpr long long kTeamQBytes = 48 * 1024;        // largest private Q-table of the team solver
 constexpr long long kTuneMinNnz = 4LL << 20;        // smallest matrix the autotuner times
 
 }  // namespace
@@ -72,6 +80,10 @@ struct Plan {
   DevBuf icwork;             // IC(0): every system's substitution words, zeroed per launch
   size_t icwork_bytes = 0;
   bool lockstep = false;
+  bool team = false;         // the team solver: one cluster per system, or the whole grid on one
+  int team_cluster = 0;      // ... CTAs of a cluster (0: the whole grid)
+  DevBuf xch;                // ... exchange words of the whole-grid team
+  size_t xch_bytes = 0;
   bool stepped = false;      // one system, one kernel per phase in a while-loop graph
   bool stepped_host = false; // ... the passes launched by the host instead (option stepped = 3)
   unsigned host_passes = 0;  // passes the host launched (stepped_host)
@@ -94,6 +106,8 @@ struct mpcg_ctx_s {
   int occ = 0;      // CTAs per SM of the solver kernel without the stream ring
   int occ_s = 0;    // ... with the stream ring (2 * kStageBytes of dynamic shared memory)
   int socc = 0, socc_s = 0;  // same for the standalone product kernel
+  int max_cluster = 0;       // largest cluster of the team solver
+  int clusters[5] = {};      // clusters of 2^i CTAs that run at a time
   int pocc[kPhaseKernels] = {}, pocc_s[kPhaseKernels] = {};  // the stepped solve's phase kernels
   std::string err;
   Plan plan;   // reused by mpcg_solve / mpcg_solve_batched / training
@@ -111,6 +125,8 @@ struct mpcg_matrix_s {
   DevBuf icf, icd;                  // IC(0) factor (fp32, one value per stored entry), diagonal positions
   DevBuf icpf, icpb;                // IC(0): rows in level order of the two substitutions
   DevBuf icof, icob;                // ... the start of each level in them
+  DevBuf icblob, icdesc;            // ... and the factor as one block per level (team solver)
+  int icring = 0, icwarps = 0;      // ... bytes of its ring, warps of the widest level (0: no blocks)
   int icwf = 0, icwb = 0;           // ... the widest level's row count
   int nlevf = 0, nlevb = 0;         // ... and the number of levels
   unsigned ic_fail = 0;             // 0: not factored or factored fine; else the factorization's error bits
@@ -418,6 +434,68 @@ mpcg_status ensure_ic0(mpcg_ctx_t ctx, mpcg_matrix_s* M, cudaStream_t s) {
     if (n) CK(ctx, cudaMemcpy(out.p, perm.data(), 4 * (size_t)n, cudaMemcpyHostToDevice));
     return MPCG_OK;
   };
+  // The team solver's form: per level a block {groups of 32 rows, quads of entries, the next block's
+  // place in the ring, bytes of a group}, then per group each lane's {row, diagonal} (row 0xffff:
+  // padding), columns and values, quad q of lane t at 32 q + t; padding entries are 0 in column n.
+  // Only for systems whose vector fits a CTA's shared memory beside a ring of blocks and whose
+  // levels are even enough not to be blown up by the padding.
+  std::vector<float> hF;
+  std::vector<unsigned char> blob;
+  std::vector<int4> desc;
+  size_t block_max = 0, groups_max = 0;
+  bool packed = n > 0 && n <= kTeamIcRows;
+  if (packed) {
+    hF.resize((size_t)std::max(nnz, 1LL));
+    CK(ctx, cudaMemcpy(hF.data(), M->icf.p, 4 * (size_t)nnz, cudaMemcpyDeviceToHost));
+  }
+  auto pack_levels = [&](int depth, bool lower) {  // lev, perm: this direction's levels and order
+    std::vector<int> start(depth + 1, 0);
+    for (int i = 0; i < n; ++i) ++start[lev[i] + 1];
+    for (int l = 0; l < depth; ++l) start[l + 1] += start[l];
+    for (int l = 0; l < depth && packed; ++l) {
+      const int cnt = start[l + 1] - start[l], ng = (cnt + 31) / 32;
+      auto first = [&](int i) { return lower ? hrp[i] : hdp[i] + 1; };
+      auto last = [&](int i) { return lower ? hdp[i] : hrp[i + 1]; };
+      int len = 0;
+      for (int x = start[l]; x < start[l + 1]; ++x) len = std::max(len, last(perm[x]) - first(perm[x]));
+      // quads of entries: one, two, or a multiple of four
+      const int quads = len <= 4 ? 1 : len <= 8 ? 2 : (len + 15) / 16 * 4;
+      const size_t group = 256 + 768 * (size_t)quads, bytes = 16 + ng * group;
+      block_max = std::max(block_max, bytes);
+      groups_max = std::max(groups_max, (size_t)ng);
+      if (3 * block_max > kTeamIcRing || blob.size() + bytes > 64ull * nnz + (1u << 20)) {
+        packed = false;
+        return;
+      }
+      const size_t at = blob.size();
+      desc.push_back(make_int4((int)(at / 16), (int)(bytes / 16), 0, 0));
+      blob.resize(at + bytes, 0);
+      unsigned char* o = blob.data() + at;
+      ((int*)o)[0] = ng;
+      ((int*)o)[1] = quads;
+      ((int*)o)[3] = (int)group;
+      for (int x = 0; x < ng * 32; ++x) {
+        const int t = x % 32;
+        unsigned char* og = o + 16 + (size_t)(x / 32) * group;
+        uint2* meta = (uint2*)og;
+        unsigned short* cols = (unsigned short*)(og + 256);
+        float* vals = (float*)(og + 256 + 256 * (size_t)quads);
+        for (int k = 0; k < 4 * quads; ++k) cols[(k / 4 * 32 + t) * 4 + k % 4] = (unsigned short)n;
+        if (x >= cnt) {
+          meta[t] = make_uint2(0xffffu, 0u);
+          continue;
+        }
+        const int i = perm[start[l] + x], e0 = first(i), e1 = last(i);
+        unsigned bits;
+        memcpy(&bits, &hF[hdp[i]], 4);
+        meta[t] = make_uint2((unsigned)i, bits);
+        for (int k = 0; k < e1 - e0; ++k) {
+          cols[(k / 4 * 32 + t) * 4 + k % 4] = (unsigned short)hci[e0 + k];
+          vals[(k / 4 * 32 + t) * 4 + k % 4] = hF[e0 + k];
+        }
+      }
+    }
+  };
   int depth = 0;
   for (int i = 0; i < n; ++i) {  // L y = r: row i reads y_j, j < i, over its lower entries
     int l = 0;
@@ -427,6 +505,7 @@ mpcg_status ensure_ic0(mpcg_ctx_t ctx, mpcg_matrix_s* M, cudaStream_t s) {
   }
   mpcg_status ls = sort_by_level(depth, M->icpf, M->icof, M->icwf, M->nlevf);
   if (ls != MPCG_OK) return ls;
+  if (packed) pack_levels(depth, true);
   depth = 0;
   for (int i = n - 1; i >= 0; --i) {  // L^T w = y: row i reads w_j, j > i, over its upper entries
     int l = 0;
@@ -436,8 +515,208 @@ mpcg_status ensure_ic0(mpcg_ctx_t ctx, mpcg_matrix_s* M, cudaStream_t s) {
   }
   ls = sort_by_level(depth, M->icpb, M->icob, M->icwb, M->nlevb);
   if (ls != MPCG_OK) return ls;
+  if (packed) pack_levels(depth, false);
+  if (packed) {
+    // places in the ring, in order from its start; a block that would cross the end goes back to the
+    // start. Block l may be written when every earlier block in its way has been consumed, and at
+    // most kTeamIcBars blocks are in flight.
+    const size_t fit = kTeamIcShared / 16 * 16 - 8 * (((size_t)n + 2) / 2);  // beside the vector
+    const int cap = (int)(std::min(std::min(kTeamIcRing, fit) & ~(size_t)15, blob.size()) / 16);
+    int at = 0;
+    for (size_t l = 0; l < desc.size(); ++l) {
+      if (at + desc[l].y > cap) at = 0;
+      desc[l].z = at;
+      at += desc[l].y;
+      int need = std::max(0, (int)l - kTeamIcBars + 1);
+      for (int j = (int)l - 1; j >= need; --j)
+        if (desc[j].z < desc[l].z + desc[l].y && desc[l].z < desc[j].z + desc[j].y) need = j + 1;
+      desc[l].w = need;
+    }
+    for (size_t l = 0; l + 1 < desc.size(); ++l)  // each block names the next one's place
+      memcpy(blob.data() + (size_t)desc[l].x * 16 + 8, &desc[l + 1].z, 4);
+    M->icring = cap * 16;
+    CK(ctx, M->icblob.ensure(blob.size()));
+    CK(ctx, M->icdesc.ensure(sizeof(int4) * desc.size()));
+    CK(ctx, cudaMemcpy(M->icblob.p, blob.data(), blob.size(), cudaMemcpyHostToDevice));
+    CK(ctx, cudaMemcpy(M->icdesc.p, desc.data(), sizeof(int4) * desc.size(), cudaMemcpyHostToDevice));
+    M->icwarps = (int)std::min<size_t>(groups_max, kTeamThreads / 32 - 2);  // (one warp waits, one copies)
+    M->bytes += (long long)blob.size();
+  }
   M->ic_ready = true;
   M->bytes += 4 * nnz + 12LL * n;
+  return MPCG_OK;
+}
+
+// Shared memory of the IC(0) substitutions of a team: the ring of level blocks and the vector.
+size_t team_ic_bytes(const mpcg_matrix_s* A) {
+  return (size_t)A->icring + 8 * (((size_t)A->dm.n + 2) / 2);
+}
+
+// CTAs of each system's team in clusters of up to `most`: its share of the places that run at a
+// time by its cost (work per iteration times the iterations it may take), to the nearest power of
+// two, and no more than one per kTeamCtaWork of work. The estimated time is the longest team's, or
+// all teams' over the places. `size` may be nullptr.
+struct TeamEstimate {
+  double time;    // in units of cost on one CTA
+  bool one_wave;  // all teams fit the places
+};
+TeamEstimate team_sizes(mpcg_ctx_t ctx, const std::vector<SysIn>& in, int most, int* size) {
+  int lg = 0;
+  while ((1 << lg) < most) ++lg;
+  const double places = std::max(1, ctx->clusters[lg]) * (double)most;
+  auto work = [&](const SysIn& s) { return (double)(s.A->dm.nnz + 4LL * s.A->dm.n + 1); };
+  auto cost = [&](const SysIn& s) { return work(s) * std::max(s.max_iter, 1); };
+  double total = 0;
+  for (const SysIn& s : in) total += cost(s);
+  double longest = 0;
+  std::vector<int> by_size(6, 0);
+  for (size_t i = 0; i < in.size(); ++i) {
+    const double share = 1.41421 * cost(in[i]) * places / total;
+    int c = 1, l = 0;
+    while (2 * c <= most && 2 * c <= share && c * (double)kTeamCtaWork < work(in[i])) c *= 2, ++l;
+    if (size) size[i] = c;
+    ++by_size[l];
+    longest = std::max(longest, cost(in[i]) / c);
+  }
+  int clusters = 0;  // teams of one size share clusters
+  for (int l = 0, c = 1; c <= most; ++l, c *= 2) clusters += (by_size[l] * c + most - 1) / most;
+  return TeamEstimate{std::max(longest, total / places), clusters <= std::max(1, ctx->clusters[lg])};
+}
+
+// The team solver takes a launch when every product of its matrices runs one of the two
+// row-length schedules, the options are those it implements, and (training) the private table
+// fits beside the vectors. Returns the CTAs per cluster, 0 for the whole grid on one system, -1
+// when another kernel takes the launch.
+int team_rule(mpcg_ctx_t ctx, const std::vector<SysIn>& in, mpcg_policy_t policy, int train) {
+  const int nsys = (int)in.size();
+  if (nsys < 1 || ctx->max_cluster < 1 || ctx->opt.variant != 0 || ctx->opt.batch_mode == 2) return -1;
+  const bool ic = ctx->opt.precond == 2;
+  const int S = ctx->opt.b_bins * ctx->opt.r_bins, joint = ctx->opt.joint ? 1 : 0;
+  const size_t table = policy->kind == 2 ? (size_t)kTeamQBytes + 4 * (size_t)visits_size(S, joint) : 0;
+  for (const SysIn& s : in) {  // the ring, the vector and the table fit a CTA's shared memory
+    const size_t need = team_ic_bytes(s.A) + table + 256;
+    if (ic && (!s.A->icwarps || need > team_max_heap())) return -1;
+  }
+  for (const SysIn& s : in)
+    for (int f = 0; f < NFMT; ++f)
+      if (s.A->dm.sched[f] != SCHED_VLOAD && s.A->dm.sched[f] != SCHED_VECTOR) return -1;
+  if (train && policy->kind == 2 && 8 * qtable_size(S, ctx->opt.nprec, joint) > kTeamQBytes) return -1;
+  if (nsys > 1) {
+    // teams when all run at a time (a cluster's places stay taken until its last team is done) and
+    // by the estimate below sooner than the lockstep kernel: per CTA 0.84 ns a unit of cost and 10 us
+    // an iteration, against 100 us an iteration and the matrices at 4 TB/s (48 systems of 1,000 to
+    // 60,000 rows, 60 iterations: 5.2 against 7.9 ms; 512 systems of 6e8 nonzeros, 5,000
+    // iterations: 71 against 10.8 s). IC(0) substitutions run in the team whenever they can.
+    const int c8 = std::min(kTeamBatchCluster, ctx->max_cluster);
+    int cluster = c8;
+    TeamEstimate e = team_sizes(ctx, in, c8, nullptr);
+    const TeamEstimate e16 = team_sizes(ctx, in, ctx->max_cluster, nullptr);
+    if (e16.time < 0.8 * e.time || (!e.one_wave && e16.one_wave)) {
+      e = e16;
+      cluster = ctx->max_cluster;
+    }
+    if (ic) return cluster;
+    if (ctx->opt.batch_mode == 1) return e.one_wave ? cluster : -1;
+    double iters = 0, total = 0;
+    for (const SysIn& s : in) {
+      iters = std::max(iters, (double)s.max_iter);
+      total += (double)s.max_iter * (s.A->dm.nnz + 4.0 * s.A->dm.n);
+    }
+    const double team = 1.2 * 0.84e-9 * e.time + 10e-6 * iters, lockstep = 100e-6 * iters + 12.0 * total / 4e12;
+    return e.one_wave && team < lockstep ? cluster : -1;
+  }
+  const long long w = in[0].A->dm.nnz + 4LL * in[0].A->dm.n;
+  return ic || w < kTeamGridWork ? ctx->max_cluster : 0;
+}
+
+// Device tables of a launch of the team solver (systems as in build_plan).
+mpcg_status build_team_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& in, mpcg_policy_t policy, int train,
+                            int trans_cap, int cluster, cudaStream_t s) {
+  const int nsys = (int)in.size();
+  pl.team = true;
+  pl.lockstep = pl.stepped = pl.stepped_host = false;
+  pl.team_cluster = cluster;
+  // teams, largest systems first (the hardware starts the next cluster where one has finished);
+  // systems that need fewer CTAs than a cluster has share one
+  std::vector<int> order(nsys);
+  std::iota(order.begin(), order.end(), 0);
+  auto cost = [&](int i) { return (in[i].A->dm.nnz + 4.0 * in[i].A->dm.n) * std::max(in[i].max_iter, 1); };
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost(a) > cost(b); });
+  std::vector<int4> ctas;
+  std::vector<int> parts_of(nsys, ctx->nsm);
+  if (cluster) {
+    team_sizes(ctx, in, cluster, parts_of.data());
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return parts_of[a] > parts_of[b]; });
+    int size = 0, used = cluster;  // team size of the cluster being filled, places taken
+    for (int i : order) {
+      const int sz = parts_of[i];
+      if (sz != size || used + sz > cluster) {
+        ctas.resize(ctas.size() + cluster, make_int4(-1, 0, 0, 0));
+        size = sz;
+        used = 0;
+      }
+      int4* c = ctas.data() + ctas.size() - cluster + used;
+      for (int r = 0; r < sz; ++r) c[r] = make_int4(i, r, sz, used);
+      used += sz;
+    }
+    CK(ctx, pl.cta_team.ensure(sizeof(int4) * ctas.size()));
+    CK(ctx, cudaMemcpyAsync(pl.cta_team.p, ctas.data(), sizeof(int4) * ctas.size(), cudaMemcpyHostToDevice, s));
+    CK(ctx, cudaStreamSynchronize(s));  // (pageable host memory)
+  }
+  const int grid = cluster ? (int)ctas.size() : ctx->nsm;
+  pl.xch_bytes = cluster ? 0 : 2 * 4 * sizeof(uint4) * (size_t)grid;
+  if (pl.xch_bytes) CK(ctx, pl.xch.ensure(pl.xch_bytes));
+  // Shared memory: the fixed part, the whole-grid exchange's values, the private table, and the
+  // vectors of the largest share of rows (even shares of nnz + 4 n; of rows half as long as the
+  // mean, as at grid boundaries, a share holds that many). A CTA whose rows exceed what was given
+  // keeps its vectors in global memory.
+  const int S = ctx->opt.b_bins * ctx->opt.r_bins, joint = ctx->opt.joint ? 1 : 0;
+  const bool table = policy->kind == 2 && 8 * qtable_size(S, ctx->opt.nprec, joint) <= kTeamQBytes;
+  const int team_q = table ? (int)qtable_size(S, ctx->opt.nprec, joint) : 0;
+  const int team_v = table ? (int)visits_size(S, joint) : 0;
+  size_t heap = 0;
+  for (int i = 0; i < nsys; ++i) {
+    const mpcg_matrix_s* A = in[i].A;
+    const int parts = parts_of[i];
+    const double w = (double)A->dm.nnz + 4.0 * A->dm.n;
+    const size_t rows =
+        std::min((size_t)A->dm.n, parts == 1 ? (size_t)A->dm.n : (size_t)(w / (parts * (4.0 + 0.5 * A->mean))) + 64);
+    const size_t icb = ctx->opt.precond == 2 ? team_ic_bytes(A) : 0;
+    size_t need = 32 * rows + icb;
+    // the columns and row bounds too where that leaves the L1 half of the SM's memory
+    const size_t idx = 4 * ((size_t)(1.3 * A->dm.nnz / parts) + rows + 64);
+    if (need + idx <= kTeamIndexHeap) need += idx;
+    heap = std::max(heap, need);
+  }
+  heap += (cluster ? 0 : 8 * 4 * (size_t)grid) + 8 * (size_t)(team_q + (team_v + 1) / 2 + 1);
+  heap = std::min((heap + 127) / 128 * 128, team_max_heap());
+  CK(ctx, pl.sys.ensure(sizeof(DevSys) * nsys));
+  CK(ctx, pl.st.ensure(sizeof(SysState) * nsys));
+  CK(ctx, pl.res.ensure(sizeof(mpcg_result) * nsys));
+  CK(ctx, pl.err.ensure(sizeof(unsigned)));
+  CK(ctx, cudaMemcpyAsync(pl.sys.p, pl.hsys.data(), sizeof(DevSys) * nsys, cudaMemcpyHostToDevice, s));
+  pl.grid = grid;
+  pl.nsys = nsys;
+  pl.nteams = 0;
+  Launch& L = pl.L;
+  memset(&L, 0, sizeof(L));
+  L.sys = pl.sys.as<DevSys>();
+  L.st = pl.st.as<SysState>();
+  L.nsys = nsys;
+  L.team_cta = pl.cta_team.as<int4>();
+  L.res = pl.res.as<mpcg_result>();
+  L.err = pl.err.as<unsigned>();
+  L.xch = pl.xch.as<uint4>();
+  L.team_heap = (int)heap;
+  L.team_q = team_q;
+  L.team_v = team_v;
+  const mpcg_status st = fill_policy(ctx, policy, L.pol);
+  if (st != MPCG_OK) return st;
+  L.opt = ctx->ov;
+  L.train = train;
+  L.ic = ctx->opt.precond == 2 ? 1 : 0;
+  L.timeout_cycles = kTimeoutCycles;
+  if (const char* t = getenv("MPCG_TIMEOUT_CYCLES")) L.timeout_cycles = atoll(t);
   return MPCG_OK;
 }
 
@@ -458,38 +737,6 @@ mpcg_status build_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& in, m
       mpcg_status st = ensure_ic0(ctx, in[i].A, s);
       if (st != MPCG_OK) return st;
     }
-  bool stream_shape = false;
-  for (int i = 0; i < nsys; ++i) stream_shape = stream_shape || uses_stream(in[i].A->dm);
-  const int grid = ctx->nsm * (stream_shape ? ctx->occ_s : ctx->occ);
-  std::vector<long long> work(nsys);
-  for (int i = 0; i < nsys; ++i) work[i] = in[i].A->dm.nnz + 4LL * in[i].A->dm.n;
-  std::vector<int> tsize;
-  std::vector<std::vector<int>> tsys;
-  schedule(work, grid, force_team, tsize, tsys);
-  const int nteams = (int)tsize.size();
-  std::vector<int> cta_team(grid, nteams), cta_rank(grid, 0), team_first(nteams + 1, 0), team_sys_off(nteams + 2, 0), team_sys_flat;
-  int c = 0;
-  for (int t = 0; t < nteams; ++t) {
-    team_first[t] = c;
-    for (int r = 0; r < tsize[t]; ++r, ++c) {
-      cta_team[c] = t;
-      cta_rank[c] = r;
-    }
-    team_sys_off[t] = (int)team_sys_flat.size();
-    for (int i : tsys[t]) team_sys_flat.push_back(i);
-  }
-  team_sys_off[nteams] = (int)team_sys_flat.size();
-  // CTAs beyond the scheduled teams form one extra empty team.
-  std::vector<int> tsize_all(tsize);
-  tsize_all.push_back(std::max(1, grid - c));
-  team_first[nteams] = c;
-  team_sys_off[nteams + 1] = team_sys_off[nteams];
-  for (int cc = c; cc < grid; ++cc) {
-    cta_team[cc] = nteams;
-    cta_rank[cc] = cc - c;
-  }
-  const int nteams_all = nteams + 1;
-
   // Work vectors: r, p, q (8 bytes per row each) and p's low-precision copy (4 bytes).
   // IC(0) adds one 64-bit word per row (value and mark of the substitutions).
   size_t wbytes = 0, mbytes = 0;
@@ -529,6 +776,10 @@ mpcg_status build_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& in, m
     d.A.icob = ic ? in[i].A->icob.as<int>() : nullptr;
     d.A.nlevf = ic ? in[i].A->nlevf : 0;
     d.A.nlevb = ic ? in[i].A->nlevb : 0;
+    d.A.icblob = ic && in[i].A->icwarps ? in[i].A->icblob.as<unsigned char>() : nullptr;
+    d.A.icdesc = in[i].A->icdesc.as<int4>();
+    d.A.icring = in[i].A->icring;
+    d.A.icwarps = in[i].A->icwarps;
     const int n = d.A.n;
     d.b = in[i].b;
     d.x = in[i].x;
@@ -557,6 +808,43 @@ mpcg_status build_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& in, m
       d.feat_cap = feat_cap;
     }
   }
+  pl.team = false;
+  if (!stepped && force_team == 0) {
+    const int cluster = team_rule(ctx, in, policy, train);
+    if (cluster >= 0) return build_team_plan(ctx, pl, in, policy, train, trans_cap, cluster, s);
+  }
+  bool stream_shape = false;
+  for (int i = 0; i < nsys; ++i) stream_shape = stream_shape || uses_stream(in[i].A->dm);
+  const int grid = ctx->nsm * (stream_shape ? ctx->occ_s : ctx->occ);
+  std::vector<long long> work(nsys);
+  for (int i = 0; i < nsys; ++i) work[i] = in[i].A->dm.nnz + 4LL * in[i].A->dm.n;
+  std::vector<int> tsize;
+  std::vector<std::vector<int>> tsys;
+  schedule(work, grid, force_team, tsize, tsys);
+  const int nteams = (int)tsize.size();
+  std::vector<int> cta_team(grid, nteams), cta_rank(grid, 0), team_first(nteams + 1, 0), team_sys_off(nteams + 2, 0), team_sys_flat;
+  int c = 0;
+  for (int t = 0; t < nteams; ++t) {
+    team_first[t] = c;
+    for (int r = 0; r < tsize[t]; ++r, ++c) {
+      cta_team[c] = t;
+      cta_rank[c] = r;
+    }
+    team_sys_off[t] = (int)team_sys_flat.size();
+    for (int i : tsys[t]) team_sys_flat.push_back(i);
+  }
+  team_sys_off[nteams] = (int)team_sys_flat.size();
+  // CTAs beyond the scheduled teams form one extra empty team.
+  std::vector<int> tsize_all(tsize);
+  tsize_all.push_back(std::max(1, grid - c));
+  team_first[nteams] = c;
+  team_sys_off[nteams + 1] = team_sys_off[nteams];
+  for (int cc = c; cc < grid; ++cc) {
+    cta_team[cc] = nteams;
+    cta_rank[cc] = cc - c;
+  }
+  const int nteams_all = nteams + 1;
+
   CK(ctx, pl.sys.ensure(sizeof(DevSys) * std::max(nsys, 1)));
   CK(ctx, pl.st.ensure(sizeof(SysState) * std::max(nsys, 1)));
   CK(ctx, pl.res.ensure(sizeof(mpcg_result) * std::max(nsys, 1)));
@@ -653,6 +941,13 @@ mpcg_status build_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& in, m
 
 // Enqueues one launch of a built plan (barrier counters and status word cleared first).
 mpcg_status enqueue_plan(mpcg_ctx_t ctx, Plan& pl, cudaStream_t s) {
+  if (pl.team) {
+    CK(ctx, cudaMemsetAsync(pl.err.p, 0, sizeof(unsigned), s));
+    if (pl.xch_bytes) CK(ctx, cudaMemsetAsync(pl.xch.p, 0, pl.xch_bytes, s));
+    cudaGetLastError();
+    CK(ctx, launch_cg_team(pl.L, pl.team_cluster, pl.grid, s));
+    return MPCG_OK;
+  }
   CK(ctx, cudaMemsetAsync(pl.bars.p, 0, sizeof(unsigned) * kBarStride * pl.nteams, s));
   CK(ctx, cudaMemsetAsync(pl.err.p, 0, sizeof(unsigned), s));
   if (pl.icwork_bytes) CK(ctx, cudaMemsetAsync(pl.icwork.p, 0, pl.icwork_bytes, s));
@@ -822,6 +1117,7 @@ mpcg_status mpcg_create(mpcg_ctx_t* out, int device, const mpcg_options* opt) {
     if (stepped_occupancy(w, &c->pocc_s[w], 2 * (size_t)kStageBytes) != cudaSuccess || c->pocc_s[w] < 1)
       return MPCG_ERR_CUDA;
   }
+  if (team_setup(&c->max_cluster, c->clusters) != cudaSuccess) return MPCG_ERR_CUDA;
   c->socc = std::min(c->socc, c->occ);
   c->socc_s = std::min(c->socc_s, c->occ_s);
   *out = c.release();
@@ -915,6 +1211,7 @@ mpcg_status mpcg_matrix_create(mpcg_ctx_t ctx, const mpcg_csr* A, mpcg_matrix_t*
   d.v8 = M->v8.as<q52_t>();
   d.rexp = M->rexp.as<short>();
   d.cols_sorted = (hf[0] & 32) ? 0 : 1;
+  d.max_row = 0;  // set with the row statistics below
   CK(ctx, launch_convert(d, M->v32.as<float>(), M->vtf.as<float>(), M->v16.as<__half>(), M->vbf.as<__nv_bfloat16>(),
                          M->v16r.as<__half>(), M->vbfr.as<__nv_bfloat16>(), M->v8.as<q52_t>(), M->rexp.as<short>(), s));
   // Jacobi: fp64 reciprocals of the diagonal, and whether every row has a positive one.
@@ -943,6 +1240,7 @@ mpcg_status mpcg_matrix_create(mpcg_ctx_t ctx, const mpcg_csr* A, mpcg_matrix_t*
   }
   M->mean = n ? sum / n : 0.0;
   M->maxr = mx;
+  d.max_row = (int)mx;
   for (int li = 0; li < 4; ++li) {
     const int tr = kThreads >> li;
     long long w = 0;

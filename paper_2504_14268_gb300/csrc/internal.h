@@ -19,6 +19,9 @@ constexpr int kNSlot = 8;           // partial sums per CTA and phase
 constexpr int kNFeat = 16;          // MLP input features
 constexpr int kMaxHidden = 128;     // MLP hidden width bound
 constexpr int kBarStride = 32;      // uint32 words between team barriers (128 bytes)
+constexpr int kTeamThreads = 1024;  // threads per CTA of the team solver
+constexpr int kTeamIcBars = 32;    // level blocks of the IC(0) substitutions in flight at most
+constexpr int kTeamMaxCluster = 16; // CTAs of a cluster team at most
 constexpr int kStageBytes = 24 * 1024;  // one stage of the stream schedule's shared-memory ring
 
 enum Sched : int { SCHED_VECTOR = 0, SCHED_STREAM = 1, SCHED_VLOAD = 2, SCHED_MERGE = 3, SCHED_XSTAGE = 4 };
@@ -43,6 +46,7 @@ struct DevMatrix {
   int lanes[8];             // lanes per row per format
   int tile_rows[8];         // stream schedule: rows per shared-memory tile (kThreads / lanes)
   int tile_bytes[8];        // stream schedule: bytes of a stage's value region (columns follow)
+  int max_row;              // nonzeros of the longest row
   int cols_sorted;          // every row's column indices strictly increase
   const double* dinv;       // Jacobi: 1 / a_ii in fp64 when the launch preconditions, else nullptr
   const float* icf;         // IC(0) factor in fp32 when the launch preconditions with it, else
@@ -54,6 +58,10 @@ struct DevMatrix {
   const int* icof;          // IC(0): start of each level in icpf (nlevf + 1 entries), then
   const int* icob;          // ... in icpb (nlevb + 1 entries)
   int nlevf, nlevb;
+  const unsigned char* icblob;  // team solver: the factor as one block per level, forward then
+  const int4* icdesc;           // backward; per block its place and size, place in the ring (16-byte
+                                // units) and the levels consumed before it may be written there
+  int icring, icwarps;          // bytes of the ring (a multiple of 16), warps of the widest level
 };
 
 // One transition of an exploration episode (Algorithm 1), recorded for the end-of-round merge.
@@ -79,7 +87,9 @@ struct DevSys {
   mpcg_iter_record* hist;   // device array or nullptr
   int hist_cap;
   int pad1;
-  double* Qpriv;            // training: lane-private copy of the tables
+  double* Qpriv;            // training: lane-private copy of the tables (team solver: the table in
+                            // shared memory, in inference too)
+  const int* vtab;          // team solver: the table's visit counts in shared memory, or nullptr
   Transition* trans;        // training: transitions of this lane's episode
   int trans_cap;
   int pad2;
@@ -185,6 +195,12 @@ struct Launch {
   int* lk_done;             // number of finished systems
   int4* lk_seg;             // [grid][nsys + 1] slices of each CTA: (system, r0, r1, partial slot)
   int* lk_nseg;             // [grid] number of slices of each CTA
+  // Team solver (team.cuh)
+  uint4* xch;               // whole-grid team: [2][grid][4] exchange words, zeroed per launch
+  int team_heap;            // bytes of shared memory behind the fixed part
+  int team_q;               // entries of the Q-table held in shared memory (0: none) ...
+  int team_v;               // ... and of its visit counts
+  const int4* team_cta;     // clusters: per CTA the system, rank, team size, first CTA of the team
 };
 
 // max over the entries a of a Q-table row that bit a of `mask` allows (the bootstrap term
@@ -247,6 +263,14 @@ cudaError_t lockstep_set_smem_limit(size_t bytes);
 cudaError_t lockstep_set_smem_limit_ic(size_t bytes);
 cudaError_t cg_occupancy(int* blocks_per_sm, size_t smem);
 size_t cg_static_smem();
+// Team solver (cg_team.cu): clusters of `cluster` CTAs holding the teams of L.team_cta, or 0: `grid`
+// CTAs as one team on system 0 (cooperative launch).
+size_t team_fixed_smem();
+size_t team_max_heap();
+cudaError_t team_setup(int* max_cluster, int resident[5]);
+cudaError_t launch_cg_team(const Launch& L, int cluster, int grid, cudaStream_t s);
+cudaError_t team_setup_ic(size_t smem_max);  // (cg_team_ic.cu)
+cudaError_t launch_cg_team_ic(const Launch& L, int cluster, int grid, size_t smem, cudaStream_t s);
 cudaError_t launch_validate(int n, long long nnz, const int* rp, const int* ci, const double* v,
                             unsigned* flags, int* bad_row, cudaStream_t s);
 cudaError_t launch_convert(const DevMatrix& A, float* v32, float* vtf, __half* v16, __nv_bfloat16* vbf,

@@ -200,18 +200,36 @@ __device__ __forceinline__ void load_bcast(const SysState* st, Smem& sm) {
 // ----------------------------------------------------------------------------------------
 // Policy (Section 4.1): state, action, reward, Q update
 // ----------------------------------------------------------------------------------------
+// In the team solver the scalar steps are out of line, one copy each: inlined at every place that
+// takes a decision they made up most of a kernel of over a megabyte, whose iterations then fetched
+// their code from L2.
+#ifndef MPCG_STEP
+#define MPCG_STEP
+#endif
 
 __device__ __forceinline__ int state_of(const OptView& o, int k, double rho) {
   int i = k / o.t_width;
   if (i > o.b_bins - 1) i = o.b_bins - 1;
   int j = 0;
-  for (int m = 1; m < o.r_bins; ++m) j += (rho <= o.thr[m]) ? 1 : 0;
+  // non-negative values order as their bit patterns (an fp64 comparison takes 64 cycles)
+  const long long rb = __double_as_longlong(rho);
+  for (int m = 1; m < o.r_bins; ++m) j += (rb <= __double_as_longlong(o.thr[m])) ? 1 : 0;
   return i * o.r_bins + j;
+}
+
+// 1 when rho lies within edge_tol (relative) of a residual-bin threshold. The fp64 division (some
+// 600 cycles) is made only for thresholds that an fp32 quotient leaves in question.
+__device__ __forceinline__ int near_bin_edge(const OptView& o, double rho) {
+  int near = 0;
+  const float r = (float)rho, lim = (float)o.edge_tol * 1.001f + 1e-5f;
+  for (int m = 1; m < o.r_bins; ++m)
+    if (fabsf(__fdividef(r, (float)o.thr[m]) - 1.f) <= lim) near |= fabs(rho / o.thr[m] - 1.0) <= o.edge_tol ? 1 : 0;
+  return near;
 }
 
 // Reward of Section 4.1, evaluated with separately rounded operations in the order
 // w1 min(-log10 rho, cap) - w2 c(p_1) - ... - w2 c(p_4) [+ w3].
-__device__ double reward_of(const OptView& o, double rho, const int* act, double tau, bool breakdown) {
+__device__ MPCG_STEP double reward_of(const OptView& o, double rho, const int* act, double tau, bool breakdown) {
   double acc;
   if (breakdown) {
     acc = -o.log_cap;
@@ -262,7 +280,7 @@ __device__ __forceinline__ void policy_draw(const Launch& L, const DevSys& S, in
 
 // Q_j(s, a_j) += lr (R + gamma max_{p in P_j} Q_j(s', p) - Q_j(s, a_j)), terminal without the max
 // term; P_j = the entries operation j may choose (op_mask).
-__device__ void q_update(double* Q, const OptView& o, const Transition& t) {
+__device__ MPCG_STEP void q_update(double* Q, const OptView& o, const Transition& t) {
   const int S = o.b_bins * o.r_bins;
   if (o.joint) {  // one entry of the joint table, bootstrap max over the allowed joint actions
     const int np4 = o.nprec * o.nprec * o.nprec * o.nprec;
@@ -287,7 +305,7 @@ __device__ void q_update(double* Q, const OptView& o, const Transition& t) {
 }
 
 // MLP forward pass by the whole CTA, fp32, weights read through the read-only path.
-__device__ void mlp_forward(const float* __restrict__ w, int H, int nout, Smem& sm) {
+__device__ MPCG_STEP void mlp_forward(const float* __restrict__ w, int H, int nout, Smem& sm) {
   const float* W1 = w;
   const float* b1 = W1 + H * kNFeat;
   const float* W2 = b1 + H;
@@ -320,7 +338,7 @@ __device__ __forceinline__ float safe_log10f(double v) { return v > 0.0 ? (float
 // the solver state): k / t_bin, -log10 max(rho, eps_min) / 16, one- and eight-step log10
 // residual ratios, log10 |alpha|, log10 |beta| (/ 8), log10 of the last true/recursive
 // residual gap, previous action indices / (nprec - 1).
-__device__ void mlp_features(const Launch& L, const DevSys& S, const SysState* st, int k, Smem& sm) {
+__device__ MPCG_STEP void mlp_features(const Launch& L, const DevSys& S, const SysState* st, int k, Smem& sm) {
   const OptView& o = L.opt;
   for (int j = 0; j < 5; ++j) sm.feat[j] = S.feat_static[j];
   const double rho = st->rho_hist[0];
@@ -338,10 +356,9 @@ __device__ void mlp_features(const Launch& L, const DevSys& S, const SysState* s
 
 // Chooses the action of iteration k in state of residual rho. Called by every thread of the
 // CTA that holds the team work; the result is left in sm.a_*.
-__device__ void choose_action(const Launch& L, const DevSys& S, SysState* st, int k, double rho, Smem& sm) {
+__device__ MPCG_STEP void choose_action(const Launch& L, const DevSys& S, SysState* st, int k, double rho, Smem& sm) {
   const OptView& o = L.opt;
   const PolicyView& P = L.pol;
-  const int s = state_of(o, k, rho);
   if (P.kind == 3 || S.feat_log) {
     if (threadIdx.x == 0) {
       mlp_features(L, S, st, k, sm);
@@ -352,6 +369,7 @@ __device__ void choose_action(const Launch& L, const DevSys& S, SysState* st, in
     if (P.kind == 3 && !st->fp64_lock) mlp_forward(P.mlp, P.H, 4 * o.nprec, sm);
   }
   if (threadIdx.x == 0) {
+    const int s = state_of(o, k, rho);
     int expl = 0;
     int jact[4] = {0, 0, 0, 0};
     if (P.kind == 2 && o.joint && !st->fp64_lock) {
@@ -370,10 +388,9 @@ __device__ void choose_action(const Launch& L, const DevSys& S, SysState* st, in
           done = true;
         }
       } else {
-        int near = 0;
-        for (int m = 1; m < o.r_bins; ++m) near |= fabs(rho / o.thr[m] - 1.0) <= o.edge_tol ? 1 : 0;
-        st->near_edge += near;
-        if (P.visits && o.fallback_fmt >= 0 && o.fallback_idx >= 0 && P.visits[s] == 0) {
+        st->near_edge += near_bin_edge(o, rho);
+        const int* vis = S.vtab ? S.vtab : P.visits;
+        if (vis && o.fallback_fmt >= 0 && o.fallback_idx >= 0 && vis[s] == 0) {
           bool all = true;
           for (int j = 0; j < 4; ++j) all = all && (((unsigned)o.op_mask[j] >> o.fallback_idx) & 1u);
           if (all) {
@@ -384,7 +401,7 @@ __device__ void choose_action(const Launch& L, const DevSys& S, SysState* st, in
       }
       if (!done) {
         const int np4 = o.nprec * o.nprec * o.nprec * o.nprec;
-        const double* row = (L.train ? S.Qpriv : P.Q) + (long long)s * np4;
+        const double* row = (L.train || S.vtab ? S.Qpriv : P.Q) + (long long)s * np4;
         int best = -1;
         for (int a = 0; a < np4; ++a)
           if (joint_allowed(a, o.nprec, o.op_mask) && (best < 0 || row[a] > row[best])) best = a;
@@ -394,58 +411,59 @@ __device__ void choose_action(const Launch& L, const DevSys& S, SysState* st, in
         }
       }
     }
-    for (int j = 0; j < 4; ++j) {
-      int fmt, act = -1;
-      if (st->fp64_lock) {
-        fmt = F64;
-      } else if (P.kind == 2 && o.joint) {
-        act = jact[j];
-        fmt = o.precs[act];
-      } else if (P.kind == 0) {
-        fmt = P.fixed[j];
-      } else if (P.kind == 1) {
-        const int row = k < P.sched_len ? k : P.sched_len - 1;
-        fmt = P.sched[row * 4 + j];
-      } else {
-        const unsigned mask = (unsigned)o.op_mask[j];
-        if (P.kind == 2) {
-          const double* Qsrc = L.train ? S.Qpriv : P.Q;
-          const double* row = Qsrc + ((long long)j * (o.b_bins * o.r_bins) + s) * o.nprec;
-          act = row_argmax(row, o.nprec, mask);
-          if (!L.train && j == 0) {  // one count per decision: rho within edge_tol of a bin edge
-            int near = 0;
-            for (int m = 1; m < o.r_bins; ++m) near |= fabs(rho / o.thr[m] - 1.0) <= o.edge_tol ? 1 : 0;
-            st->near_edge += near;
-          }
-          if (!L.train && P.visits && o.fallback_fmt >= 0 && o.fallback_idx >= 0 && ((mask >> o.fallback_idx) & 1u) &&
-              P.visits[j * (o.b_bins * o.r_bins) + s] == 0)
-            act = o.fallback_idx;
-        } else {
-          int b = -1;
-          for (int a = 0; a < o.nprec; ++a)
-            if ((mask >> a) & 1u)
-              if (b < 0 || sm.out[j * o.nprec + a] > sm.out[j * o.nprec + b]) b = a;
-          act = b;
-        }
-        if (L.train) {
-          double u;
-          unsigned pick;
-          policy_draw(L, S, k, j, u, pick);
-          if (u < L.eps) {
-            act = kth_allowed(mask, (int)(pick % (unsigned)__popc(mask)));
-            expl = 1;
-          }
-        }
-        fmt = o.precs[act];
-      }
-      if (act < 0)
-        for (int a = 0; a < o.nprec; ++a)
-          if (o.precs[a] == fmt) { act = a; break; }
-      sm.a_fmt[j] = fmt;
-      sm.a_act[j] = act;
-    }
     sm.a_expl = expl;
     sm.a_state = s;
+    for (int j = 0; j < 4; ++j) sm.a_act[j] = jact[j];
+  }
+  __syncthreads();
+  if (threadIdx.x < 4) {  // one thread per operation
+    const int j = threadIdx.x;
+    const int s = sm.a_state;
+    int fmt, act = -1;
+    if (st->fp64_lock) {
+      fmt = F64;
+    } else if (P.kind == 2 && o.joint) {
+      act = sm.a_act[j];
+      fmt = o.precs[act];
+    } else if (P.kind == 0) {
+      fmt = P.fixed[j];
+    } else if (P.kind == 1) {
+      const int row = k < P.sched_len ? k : P.sched_len - 1;
+      fmt = P.sched[row * 4 + j];
+    } else {
+      const unsigned mask = (unsigned)o.op_mask[j];
+      if (P.kind == 2) {
+        const double* Qsrc = L.train || S.vtab ? S.Qpriv : P.Q;
+        const int* vis = S.vtab ? S.vtab : P.visits;
+        const double* row = Qsrc + ((long long)j * (o.b_bins * o.r_bins) + s) * o.nprec;
+        act = row_argmax(row, o.nprec, mask);
+        if (!L.train && j == 0) st->near_edge += near_bin_edge(o, rho);  // one count per decision
+        if (!L.train && vis && o.fallback_fmt >= 0 && o.fallback_idx >= 0 && ((mask >> o.fallback_idx) & 1u) &&
+            vis[j * (o.b_bins * o.r_bins) + s] == 0)
+          act = o.fallback_idx;
+      } else {
+        int b = -1;
+        for (int a = 0; a < o.nprec; ++a)
+          if ((mask >> a) & 1u)
+            if (b < 0 || sm.out[j * o.nprec + a] > sm.out[j * o.nprec + b]) b = a;
+        act = b;
+      }
+      if (L.train) {
+        double u;
+        unsigned pick;
+        policy_draw(L, S, k, j, u, pick);
+        if (u < L.eps) {
+          act = kth_allowed(mask, (int)(pick % (unsigned)__popc(mask)));
+          sm.a_expl = 1;
+        }
+      }
+      fmt = o.precs[act];
+    }
+    if (act < 0)
+      for (int a = 0; a < o.nprec; ++a)
+        if (o.precs[a] == fmt) { act = a; break; }
+    sm.a_fmt[j] = fmt;
+    sm.a_act[j] = act;
   }
   __syncthreads();
 }
@@ -602,7 +620,7 @@ __device__ __forceinline__ unsigned stamp(SysState* st) {
   return d > 0xffffffffull ? 0xffffffffu : (unsigned)d;
 }
 
-__device__ void write_record(const DevSys& S, SysState* st, int flags, double rho, double sigma, double beta,
+__device__ MPCG_STEP void write_record(const DevSys& S, SysState* st, int flags, double rho, double sigma, double beta,
                              double reward) {
   const int k = st->k;
   if (S.hist && k < S.hist_cap) {
@@ -627,7 +645,7 @@ __device__ void write_record(const DevSys& S, SysState* st, int flags, double rh
   }
 }
 
-__device__ void push_transition(const Launch& L, const DevSys& S, SysState* st, int s_next, double R,
+__device__ MPCG_STEP void push_transition(const Launch& L, const DevSys& S, SysState* st, int s_next, double R,
                                 int terminal) {
   if (!L.train) return;
   Transition t;
@@ -659,7 +677,7 @@ __device__ __forceinline__ bool restart_ok(const Launch& L, const SysState* st) 
 }
 
 // After the initial phase: ||b||, rho_0, sigma_0 = r_0^T r_0, action of iteration 0.
-__device__ void step_init(const Launch& L, const DevSys& S, SysState* st, double bb, double rr, double sig,
+__device__ MPCG_STEP void step_init(const Launch& L, const DevSys& S, SysState* st, double bb, double rr, double sig,
                           Smem& sm) {
   if (threadIdx.x == 0) {
     const double bnorm = sqrt(bb);
@@ -720,7 +738,7 @@ __device__ void step_init(const Launch& L, const DevSys& S, SysState* st, double
 // After phase A: nu = fl_p3(sum), alpha = sigma / nu, curvature breakdown test.
 __device__ void step_A(const Launch& L, const DevSys& S, SysState* st, double nu_sum) {
   if (threadIdx.x != 0) return;
-  st->ns_a = stamp(st);
+  st->ns_a = S.hist ? stamp(st) : 0u;  // only the records show the phase times
   st->ns_b = 0;
   const int p3 = st->fmt[2];
   const double nu = (p3 == F64) ? nu_sum : round_fmt(nu_sum, p3);
@@ -754,7 +772,7 @@ __device__ void step_A(const Launch& L, const DevSys& S, SysState* st, double nu
 
 // Continues after the residual of iteration k is known (recursive, or replaced when
 // `replaced`): sigma_{k+1}, beta_k (0 after a replacement), reward, next state and action.
-__device__ void continue_step(const Launch& L, const DevSys& S, SysState* st, double rho_new, double sig_sum,
+__device__ MPCG_STEP void continue_step(const Launch& L, const DevSys& S, SysState* st, double rho_new, double sig_sum,
                               int replaced, Smem& sm) {
   if (threadIdx.x == 0) {
     sm.need_action = 0;
@@ -814,7 +832,7 @@ __device__ void continue_step(const Launch& L, const DevSys& S, SysState* st, do
 // (from the recurrence, or recomputed when `replaced`): record, reward, transition, next state
 // and action. gamma and alpha of iteration k become the recurrence's previous values; a
 // replaced residual restarts the recurrence (beta = 0 next).
-__device__ void continue_sr(const Launch& L, const DevSys& S, SysState* st, double rho_new, int replaced, Smem& sm) {
+__device__ MPCG_STEP void continue_sr(const Launch& L, const DevSys& S, SysState* st, double rho_new, int replaced, Smem& sm) {
   if (threadIdx.x == 0) {
     sm.need_action = 0;
     const int k = st->k;
@@ -857,7 +875,7 @@ __device__ void continue_sr(const Launch& L, const DevSys& S, SysState* st, doub
 // at a restart), alpha = gamma / nu; breakdown tests as after phase A; the next residual norm
 // rr - 2 alpha (r.w + beta r.s) + alpha^2 (w.w + 2 beta w.s + beta^2 s.s) (clamped at 0) and the
 // stopping tests as after phase B. dots = r.r, r.w, r.s, w.w, w.s, s.s (fp64 sums).
-__device__ void step_W(const Launch& L, const DevSys& S, SysState* st, double gsum, double dsum, const double* dots,
+__device__ MPCG_STEP void step_W(const Launch& L, const DevSys& S, SysState* st, double gsum, double dsum, const double* dots,
                        Smem& sm) {
   if (threadIdx.x == 0) {
     st->ns_a = stamp(st);
@@ -939,7 +957,7 @@ __device__ void step_W(const Launch& L, const DevSys& S, SysState* st, double gs
 // After phase B: rho_{k+1} of the recursive residual, stopping tests.
 __device__ void step_B(const Launch& L, const DevSys& S, SysState* st, double rr, double sig_sum, Smem& sm) {
   if (threadIdx.x == 0) {
-    st->ns_b = stamp(st);
+    st->ns_b = S.hist ? stamp(st) : 0u;
     sm.need_action = 0;
     const double rho_rec = sqrt(rr) / st->bnorm;
     const OptView& o = L.opt;
@@ -971,14 +989,15 @@ __device__ void step_B(const Launch& L, const DevSys& S, SysState* st, double rr
       st->mode = M_X_THEN_DONE;
     } else {
       sm.flag = 1;
+      sm.tmp = rho_rec;  // (one thread's square root and division: fp64 runs 2 lanes a cycle per SM)
     }
   }
   __syncthreads();
-  if (sm.flag) continue_step(L, S, st, sqrt(rr) / st->bnorm, sig_sum, 0, sm);
+  if (sm.flag) continue_step(L, S, st, sm.tmp, sig_sum, 0, sm);
 }
 
 // After a residual recomputation inside the iteration (phase T).
-__device__ void step_T(const Launch& L, const DevSys& S, SysState* st, double rr, double sig_sum, Smem& sm) {
+__device__ MPCG_STEP void step_T(const Launch& L, const DevSys& S, SysState* st, double rr, double sig_sum, Smem& sm) {
   if (threadIdx.x == 0) {
     const double rho_t = sqrt(rr) / st->bnorm;
     const double rho_rec = st->rho_true;
@@ -1011,18 +1030,19 @@ __device__ void step_T(const Launch& L, const DevSys& S, SysState* st, double rr
       st->mode = M_DONE;
     } else {
       sm.flag = 1;
+      sm.tmp = rho_t;
     }
   }
   __syncthreads();
   if (sm.flag) {
-    if (L.opt.variant) continue_sr(L, S, st, sqrt(rr) / st->bnorm, 1, sm);
-    else continue_step(L, S, st, sqrt(rr) / st->bnorm, sig_sum, 1, sm);
+    if (L.opt.variant) continue_sr(L, S, st, sm.tmp, 1, sm);
+    else continue_step(L, S, st, sm.tmp, sig_sum, 1, sm);
   }
 }
 
 // After the fp64 restart's residual recomputation (r = b - A x, p = r): iteration k counts
 // as done; sigma = ||r||^2, every later operation in fp64; stop test as after any iteration.
-__device__ void step_restart(const Launch& L, const DevSys& S, SysState* st, double rr, double sig, Smem& sm) {
+__device__ MPCG_STEP void step_restart(const Launch& L, const DevSys& S, SysState* st, double rr, double sig, Smem& sm) {
   if (threadIdx.x == 0) {
     sm.need_action = 0;
     const double rho = sqrt(rr) / st->bnorm;
@@ -1066,7 +1086,7 @@ __device__ void step_restart(const Launch& L, const DevSys& S, SysState* st, dou
   }
 }
 
-__device__ void step_final(const Launch& L, const DevSys& S, SysState* st, int sid, double rr) {
+__device__ MPCG_STEP void step_final(const Launch& L, const DevSys& S, SysState* st, int sid, double rr) {
   if (threadIdx.x != 0) return;
   if (!st->true_known) st->rho_true = st->bnorm > 0.0 ? sqrt(rr) / st->bnorm : 0.0;
   mpcg_result res;
@@ -1105,10 +1125,10 @@ __device__ __forceinline__ bool team_step(const Launch& L, const TeamCtx& T, Sys
 
 // Stage-C stamp: phase C of the finished iteration closes at this barrier.
 __device__ __forceinline__ void stamp_c(const DevSys& S, SysState* st) {
-  if (threadIdx.x == 0) {
+  if (S.hist && threadIdx.x == 0) {
     const unsigned d = stamp(st);
     const int kd = st->k - 1;
-    if (S.hist && kd >= 0 && kd < S.hist_cap) S.hist[kd].ns_c = d;
+    if (kd >= 0 && kd < S.hist_cap) S.hist[kd].ns_c = d;
   }
 }
 

@@ -140,21 +140,23 @@ struct RowAcc {
       s = fmaf(af, xf, s);
     }
   }
+  // One butterfly step of the lanes' accumulators.
+  __device__ __forceinline__ void step(unsigned mask, int o) {
+    const float so = __shfl_xor_sync(mask, s, o);
+    if constexpr (COMP) {
+      const float co = __shfl_xor_sync(mask, c, o), ao = __shfl_xor_sync(mask, a, o);
+      float t;
+      two_sum(s, so, s, t);
+      c = __fadd_rn(__fadd_rn(c, co), t);
+      a = __fadd_rn(__fadd_rn(a, ao), fabsf(t));
+    } else {
+      s += so;
+    }
+  }
   template <int K>
   __device__ __forceinline__ void reduce(unsigned mask) {
 #pragma unroll
-    for (int o = K / 2; o > 0; o >>= 1) {
-      const float so = __shfl_xor_sync(mask, s, o);
-      if constexpr (COMP) {
-        const float co = __shfl_xor_sync(mask, c, o), ao = __shfl_xor_sync(mask, a, o);
-        float t;
-        two_sum(s, so, s, t);
-        c = __fadd_rn(__fadd_rn(c, co), t);
-        a = __fadd_rn(__fadd_rn(a, ao), fabsf(t));
-      } else {
-        s += so;
-      }
-    }
+    for (int o = K / 2; o > 0; o >>= 1) step(mask, o);
   }
   // Adds another partial accumulation of the same row (the cross-warp step of a row summed
   // by the whole CTA).
@@ -171,6 +173,11 @@ struct RowAcc {
   // Row sum rounded onto p1 (fp32 result). `exact` recomputes the row in fp64 when needed.
   template <class Exact>
   __device__ __forceinline__ float rounded(int p1, int len, Exact&& exact) const {
+    return rounded(p1, len, exact, [&] { return slow_round(p1, exact()); });
+  }
+  // ... with `redo` giving the exactly rounded value where the bound leaves the rounding open
+  template <class Exact, class Redo>
+  __device__ __forceinline__ float rounded(int p1, int len, Exact&&, Redo&& redo) const {
     if constexpr (!COMP) {
       return s;
     } else {
@@ -191,7 +198,7 @@ struct RowAcc {
       const float d = __fadd_rn(__fsub_rn(hi, r), lo);
       const float slack = fabsf(d) * 1.2e-7f;
       if (d + err + slack < above && -d + err + slack < below) return r;
-      return slow_round(p1, exact());
+      return redo();
     }
   }
   __device__ static __noinline__ float slow_round(int p1, double v) { return round_d2f(v, p1); }
@@ -202,10 +209,11 @@ struct RowAcc<double, false> {
   double s = 0.0, c = 0.0, a = 0.0;  // c and a unused (fp64 accumulation)
   __device__ __forceinline__ void add(double av, double x) { s = fma(av, x, s); }
   __device__ __forceinline__ void merge(double os, double, double) { s += os; }
+  __device__ __forceinline__ void step(unsigned mask, int o) { s += __shfl_xor_sync(mask, s, o); }
   template <int K>
   __device__ __forceinline__ void reduce(unsigned mask) {
 #pragma unroll
-    for (int o = K / 2; o > 0; o >>= 1) s += __shfl_xor_sync(mask, s, o);
+    for (int o = K / 2; o > 0; o >>= 1) step(mask, o);
   }
 };
 
