@@ -2029,8 +2029,7 @@ mpcg_status mpcg_mlp_loss_grad(mpcg_ctx_t ctx, const float* params, int64_t B, c
   cudaSetDevice(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
   const long long np = mlp_nparams_dev(o.mlp_hidden, o.nprec);
-  const int chunk = 32;
-  const int nparts = (int)((B + chunk - 1) / chunk);
+  const int nparts = (int)((B + kMlpChunk - 1) / kMlpChunk);
   DevBuf dw, df, da, dy, dpart, dl, dg, dloss;
   CK(ctx, dw.ensure(sizeof(float) * np));
   CK(ctx, df.ensure(sizeof(float) * kNFeat * B));
@@ -2045,8 +2044,8 @@ mpcg_status mpcg_mlp_loss_grad(mpcg_ctx_t ctx, const float* params, int64_t B, c
   CK(ctx, cudaMemcpyAsync(da.p, acts, sizeof(int) * 4 * B, cudaMemcpyHostToDevice, s));
   CK(ctx, cudaMemcpyAsync(dy.p, y, sizeof(float) * 4 * B, cudaMemcpyHostToDevice, s));
   CK(ctx, launch_mlp_grad(dw.as<float>(), nullptr, o.mlp_hidden, o.nprec, df.as<float>(), nullptr, da.as<int>(), nullptr,
-                          nullptr, dy.as<float>(), nullptr, (int)B, chunk, (float)o.gamma, op_masks(o),
-                          dpart.as<float>(), dl.as<double>(), s));
+                          nullptr, dy.as<float>(), 0, 0, 0, (int)B, (float)o.gamma, op_masks(o), dpart.as<float>(),
+                          dl.as<double>(), s));
   CK(ctx, launch_mlp_reduce_adam(dpart.as<float>(), nparts, np, dg.as<float>(), nullptr, nullptr, nullptr, 0, 0.f,
                                  dl.as<double>(), dloss.as<double>(), s));
   CK(ctx, cudaMemcpyAsync(grad, dg.p, sizeof(float) * np, cudaMemcpyDeviceToHost, s));
@@ -2071,8 +2070,7 @@ mpcg_status mpcg_mlp_train(mpcg_ctx_t ctx, mpcg_policy_t P, const mpcg_transitio
   cudaSetDevice(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
   const long long np = mlp_nparams_dev(o.mlp_hidden, o.nprec);
-  const int chunk = 32;
-  const int nparts = (batch + chunk - 1) / chunk;
+  const int nparts = (batch + kMlpChunk - 1) / kMlpChunk;
   std::vector<float> hF((size_t)kNFeat * count), hFn((size_t)kNFeat * count), hR(count);
   std::vector<int> hA((size_t)4 * count), hD(count);
   for (int64_t i = 0; i < count; ++i) {
@@ -2082,7 +2080,7 @@ mpcg_status mpcg_mlp_train(mpcg_ctx_t ctx, mpcg_policy_t P, const mpcg_transitio
     hR[i] = data[i].reward;
     hD[i] = data[i].done;
   }
-  DevBuf dF, dFn, dA, dR, dD, dwt, dm, dv, didx, dpart, dl, dloss;
+  DevBuf dF, dFn, dA, dR, dD, dwt, dm, dv, dpart, dl, dloss;
   CK(ctx, dF.ensure(sizeof(float) * hF.size()));
   CK(ctx, dFn.ensure(sizeof(float) * hFn.size()));
   CK(ctx, dA.ensure(sizeof(int) * hA.size()));
@@ -2091,7 +2089,6 @@ mpcg_status mpcg_mlp_train(mpcg_ctx_t ctx, mpcg_policy_t P, const mpcg_transitio
   CK(ctx, dwt.ensure(sizeof(float) * np));
   CK(ctx, dm.ensure(sizeof(float) * np));
   CK(ctx, dv.ensure(sizeof(float) * np));
-  CK(ctx, didx.ensure(sizeof(long long) * batch));
   CK(ctx, dpart.ensure(sizeof(float) * np * nparts));
   CK(ctx, dl.ensure(sizeof(double) * nparts));
   CK(ctx, dloss.ensure(sizeof(double) * steps));
@@ -2104,10 +2101,9 @@ mpcg_status mpcg_mlp_train(mpcg_ctx_t ctx, mpcg_policy_t P, const mpcg_transitio
   CK(ctx, cudaMemsetAsync(dv.p, 0, sizeof(float) * np, s));
   CK(ctx, cudaMemcpyAsync(dwt.p, P->mlp.p, sizeof(float) * np, cudaMemcpyDeviceToDevice, s));
   for (int t = 1; t <= steps; ++t) {
-    CK(ctx, launch_mlp_sample(didx.as<long long>(), batch, count, seed, (unsigned long long)t, s));
     CK(ctx, launch_mlp_grad(P->mlp.as<float>(), dwt.as<float>(), o.mlp_hidden, o.nprec, dF.as<float>(), dFn.as<float>(),
-                            dA.as<int>(), dR.as<float>(), dD.as<int>(), nullptr, didx.as<long long>(), batch, chunk,
-                            (float)o.gamma, op_masks(o), dpart.as<float>(), dl.as<double>(), s));
+                            dA.as<int>(), dR.as<float>(), dD.as<int>(), nullptr, count, seed, (unsigned long long)t,
+                            batch, (float)o.gamma, op_masks(o), dpart.as<float>(), dl.as<double>(), s));
     CK(ctx, launch_mlp_reduce_adam(dpart.as<float>(), nparts, np, nullptr, P->mlp.as<float>(), dm.as<float>(),
                                    dv.as<float>(), t, lr, dl.as<double>(), dloss.as<double>() + (t - 1), s));
     if (t % target_sync == 0)

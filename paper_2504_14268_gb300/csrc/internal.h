@@ -282,16 +282,17 @@ cudaError_t mlp_set_smem_limit(size_t bytes);
 struct OpMask {
   unsigned m[4];
 };
+constexpr int kMlpChunk = 32;  // samples per CTA (and partial gradient)
+// Gradient and loss partials of a minibatch of B samples: transitions drawn for step t from `count`
+// (count > 0) or the first B.
 cudaError_t launch_mlp_grad(const float* w, const float* wt, int H, int nprec, const float* feats,
                             const float* feats_next, const int* acts, const float* rew, const int* done, const float* y,
-                            const long long* idx, int B, int chunk, float gamma, OpMask mask, float* part,
-                            double* lpart, cudaStream_t s);
+                            long long count, unsigned long long seed, unsigned long long t, int B, float gamma,
+                            OpMask mask, float* part, double* lpart, cudaStream_t s);
 cudaError_t launch_mlp_targets(const float* wt, int H, int nprec, const float* feats_next, const float* rew,
                                const int* done, int B, float gamma, OpMask mask, float* y, cudaStream_t s);
 cudaError_t launch_mlp_reduce_adam(const float* part, int nparts, long long np, float* grad, float* w, float* m,
                                    float* v, int t, float lr, const double* lpart, double* loss, cudaStream_t s);
-cudaError_t launch_mlp_sample(long long* idx, int B, long long count, unsigned long long seed, unsigned long long t,
-                              cudaStream_t s);
 // IC(0) factorization in fp32 (sync-free: one thread per row, rows in increasing order per
 // thread, each row waiting on the completion marks of the rows it depends on; all CTAs
 // resident, cooperative launch). err bits: 1 breakdown, 2 unusable pattern, 4 time limit.
