@@ -568,19 +568,24 @@ TeamEstimate team_sizes(mpcg_ctx_t ctx, const std::vector<SysIn>& in, int most, 
   auto cost = [&](const SysIn& s) { return work(s) * std::max(s.max_iter, 1); };
   double total = 0;
   for (const SysIn& s : in) total += cost(s);
-  double longest = 0;
-  std::vector<int> by_size(6, 0);
-  for (size_t i = 0; i < in.size(); ++i) {
-    const double share = 1.41421 * cost(in[i]) * places / total;
-    int c = 1, l = 0;
-    while (2 * c <= most && 2 * c <= share && c * (double)kTeamCtaWork < work(in[i])) c *= 2, ++l;
-    if (size) size[i] = c;
-    ++by_size[l];
-    longest = std::max(longest, cost(in[i]) / c);
+  // the nearest powers of two; smaller teams (down to half) when that lets all of them run at a time
+  TeamEstimate e{0.0, false};
+  for (double f = 1.41421; f > 0.6 && !e.one_wave; f *= 0.9) {
+    double longest = 0;
+    std::vector<int> by_size(6, 0);
+    for (size_t i = 0; i < in.size(); ++i) {
+      const double share = f * cost(in[i]) * places / total;
+      int c = 1, l = 0;
+      while (2 * c <= most && 2 * c <= share && c * (double)kTeamCtaWork < work(in[i])) c *= 2, ++l;
+      if (size) size[i] = c;
+      ++by_size[l];
+      longest = std::max(longest, cost(in[i]) / c);
+    }
+    int clusters = 0;  // teams of one size share clusters
+    for (int l = 0, c = 1; c <= most; ++l, c *= 2) clusters += (by_size[l] * c + most - 1) / most;
+    e = TeamEstimate{std::max(longest, total / places), clusters <= std::max(1, ctx->clusters[lg])};
   }
-  int clusters = 0;  // teams of one size share clusters
-  for (int l = 0, c = 1; c <= most; ++l, c *= 2) clusters += (by_size[l] * c + most - 1) / most;
-  return TeamEstimate{std::max(longest, total / places), clusters <= std::max(1, ctx->clusters[lg])};
+  return e;
 }
 
 // The team solver takes a launch when every product of its matrices runs one of the two
@@ -591,6 +596,9 @@ int team_rule(mpcg_ctx_t ctx, const std::vector<SysIn>& in, mpcg_policy_t policy
   const int nsys = (int)in.size();
   if (nsys < 1 || ctx->max_cluster < 1 || ctx->opt.variant != 0 || ctx->opt.batch_mode == 2) return -1;
   const bool ic = ctx->opt.precond == 2;
+  // Training with IC(0) stays with the lockstep kernel: a learner that meets near-equal actions keeps
+  // one or the other by the last bits of the residual, and there a seed gives the same table as ever.
+  if (train && ic) return -1;
   const int S = ctx->opt.b_bins * ctx->opt.r_bins, joint = ctx->opt.joint ? 1 : 0;
   const size_t table = policy->kind == 2 ? (size_t)kTeamQBytes + 4 * (size_t)visits_size(S, joint) : 0;
   for (const SysIn& s : in) {  // the ring, the vector and the table fit a CTA's shared memory
@@ -605,8 +613,8 @@ int team_rule(mpcg_ctx_t ctx, const std::vector<SysIn>& in, mpcg_policy_t policy
     // teams when all run at a time (a cluster's places stay taken until its last team is done) and
     // by the estimate below sooner than the lockstep kernel: per CTA 0.84 ns a unit of cost and 10 us
     // an iteration, against 100 us an iteration and the matrices at 4 TB/s (48 systems of 1,000 to
-    // 60,000 rows, 60 iterations: 5.2 against 7.9 ms; 512 systems of 6e8 nonzeros, 5,000
-    // iterations: 71 against 10.8 s). IC(0) substitutions run in the team whenever they can.
+    // 60,000 rows, 60 iterations: 5.6 against 7.6 ms; 512 systems of 6e8 nonzeros, 5,000
+    // iterations: 71 against 10.7 s). IC(0) substitutions run in the team whenever they can.
     const int c8 = std::min(kTeamBatchCluster, ctx->max_cluster);
     int cluster = c8;
     TeamEstimate e = team_sizes(ctx, in, c8, nullptr);
