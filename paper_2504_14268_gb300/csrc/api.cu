@@ -55,6 +55,7 @@ bool is_device_ptr(const void* p) {
 }
 
 constexpr long long kTimeoutCycles = 4000000000ll;  // about two seconds at 2 GHz per wait
+constexpr double kTileMinMean = 14.0;              // mean row length from which warp tiles pay
 constexpr int kTeamBatchCluster = 8;               // cluster of a batch's teams
 constexpr long long kTeamCtaWork = 8192;           // a team has a CTA per so much work (nnz + 4 n)
 constexpr long long kTeamGridWork = 160 * 1000;    // from here a single system takes the whole grid
@@ -106,6 +107,7 @@ struct mpcg_ctx_s {
   int occ = 0;      // CTAs per SM of the solver kernel without the stream ring
   int occ_s = 0;    // ... with the stream ring (2 * kStageBytes of dynamic shared memory)
   int socc = 0, socc_s = 0;  // same for the standalone product kernel
+  int socc_t = 0, pocc_t = 0;  // the standalone and the stepped product kernel with warp tiles
   int max_cluster = 0;       // largest cluster of the team solver
   int clusters[5] = {};      // clusters of 2^i CTAs that run at a time
   int pocc[kPhaseKernels] = {}, pocc_s[kPhaseKernels] = {};  // the stepped solve's phase kernels
@@ -871,12 +873,16 @@ mpcg_status build_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& in, m
   pl.stepped = stepped;
   pl.stepped_host = false;
   int pgrid = 0;
+  bool tiles = false;
   if (stepped) {
     for (int w = 0; w < kPhaseKernels; ++w) {
       pl.sgrid[w] = ctx->nsm * (stream_shape ? ctx->pocc_s[w] : ctx->pocc[w]);
       pgrid = std::max(pgrid, pl.sgrid[w]);
     }
     pl.ssmem = stream_shape ? 2 * (size_t)kStageBytes : 0;
+    // a fixed policy with fp64 products (the other formats are faster from direct loads, see spmv_tile)
+    tiles = in[0].A->dm.tile && in[0].A->dm.sched[F64] == SCHED_VLOAD && policy->kind == 0 && policy->fixed[0] == F64;
+    if (tiles) pl.sgrid[0] = ctx->nsm * ctx->pocc_t;
     CK(ctx, pl.lk_done.ensure(sizeof(int)));
   }
   CK(ctx, pl.partials.ensure(sizeof(double) * kNSlot * (size_t)(std::max(grid, pgrid) + (pl.lockstep ? nsys : 0))));
@@ -929,6 +935,7 @@ mpcg_status build_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& in, m
   L.opt = ctx->ov;
   L.train = train;
   L.stream_stage = stream_shape ? kStageBytes : 0;
+  L.tile = tiles ? 1 : 0;
   L.timeout_cycles = kTimeoutCycles;
   if (const char* t = getenv("MPCG_TIMEOUT_CYCLES")) L.timeout_cycles = atoll(t);
   L.lockstep = pl.lockstep ? 1 : 0;
@@ -1125,6 +1132,8 @@ mpcg_status mpcg_create(mpcg_ctx_t* out, int device, const mpcg_options* opt) {
     if (stepped_occupancy(w, &c->pocc_s[w], 2 * (size_t)kStageBytes) != cudaSuccess || c->pocc_s[w] < 1)
       return MPCG_ERR_CUDA;
   }
+  if (spmv_tile_occupancy(&c->socc_t) != cudaSuccess || c->socc_t < 1) return MPCG_ERR_CUDA;
+  if (stepped_tile_occupancy(&c->pocc_t) != cudaSuccess || c->pocc_t < 1) return MPCG_ERR_CUDA;
   if (team_setup(&c->max_cluster, c->clusters) != cudaSuccess) return MPCG_ERR_CUDA;
   c->socc = std::min(c->socc, c->occ);
   c->socc_s = std::min(c->socc_s, c->occ_s);
@@ -1255,6 +1264,7 @@ mpcg_status mpcg_matrix_create(mpcg_ctx_t ctx, const mpcg_csr* A, mpcg_matrix_t*
     for (int i = 0; i < n; ++i) w = std::max(w, (long long)hrp[std::min(i + tr, n)] - hrp[i]);
     M->win[li] = w;
   }
+  d.tile = M->mean >= kTileMinMean && M->win[3] <= kTileEntries ? 1 : 0;
   M->cv = (n && M->mean > 0) ? std::sqrt(std::max(0.0, sq / n - M->mean * M->mean)) / M->mean : 0.0;
   // Static features of the MLP policy: log10(n) / 8, mean nnz per row / 64,
   // log10(max a_ii / min a_ii) / 16, log10(max_i sum_j |a_ij| / a_ii) / 16, and the fraction
@@ -1400,7 +1410,8 @@ mpcg_status mpcg_spmv(mpcg_ctx_t ctx, mpcg_matrix_t A, int32_t fmt, const double
   // The launch shape the solver uses for this matrix: with the stream ring when any format
   // of the matrix uses the stream schedule.
   const bool stream_shape = A->force_stream_shape || uses_stream(A->dm);
-  const int grid = ctx->nsm * (stream_shape ? ctx->occ_s : ctx->occ);
+  const bool tile = fmt == F64 && A->dm.tile && A->dm.sched[F64] == SCHED_VLOAD;
+  const int grid = ctx->nsm * (tile ? ctx->socc_t : stream_shape ? ctx->occ_s : ctx->occ);
   const int stage = stream_shape ? kStageBytes : 0;
   CK(ctx, ctx->spmv_err.ensure(sizeof(unsigned)));
   CK(ctx, cudaMemsetAsync(ctx->spmv_err.p, 0, sizeof(unsigned), s));
@@ -1408,9 +1419,9 @@ mpcg_status mpcg_spmv(mpcg_ctx_t ctx, mpcg_matrix_t A, int32_t fmt, const double
   cudaEvent_t e0, e1;
   CK(ctx, cudaEventCreate(&e0));
   CK(ctx, cudaEventCreate(&e1));
-  CK(ctx, launch_spmv_only(S, fmt, grid, stage, ctx->spmv_err.as<unsigned>(), s));  // warm-up
+  CK(ctx, launch_spmv_only(S, fmt, grid, stage, tile, ctx->spmv_err.as<unsigned>(), s));  // warm-up
   CK(ctx, cudaEventRecord(e0, s));
-  for (int r = 0; r < reps; ++r) CK(ctx, launch_spmv_only(S, fmt, grid, stage, ctx->spmv_err.as<unsigned>(), s));
+  for (int r = 0; r < reps; ++r) CK(ctx, launch_spmv_only(S, fmt, grid, stage, tile, ctx->spmv_err.as<unsigned>(), s));
   CK(ctx, cudaEventRecord(e1, s));
   CK(ctx, launch_from_q(S.q, A->dm.rexp, y, n, fmt, s));
   CK(ctx, cudaStreamSynchronize(s));

@@ -19,6 +19,9 @@ constexpr int kNSlot = 8;           // partial sums per CTA and phase
 constexpr int kNFeat = 16;          // MLP input features
 constexpr int kMaxHidden = 128;     // MLP hidden width bound
 constexpr int kBarStride = 32;      // uint32 words between team barriers (128 bytes)
+constexpr int kTileEntries = 896;   // nonzeros of a warp's tile (32 rows) of the vector-load schedule
+constexpr int kTileWarpBytes = 4 * (kTileEntries + 8) + 8 * (kTileEntries + 2);  // columns, fp64 values
+constexpr int kTileBytes = kTileWarpBytes * (kThreads / 32);
 constexpr int kTeamThreads = 1024;  // threads per CTA of the team solver
 constexpr int kTeamIcBars = 32;    // level blocks of the IC(0) substitutions in flight at most
 constexpr int kTeamMaxCluster = 16; // CTAs of a cluster team at most
@@ -47,6 +50,7 @@ struct DevMatrix {
   int tile_rows[8];         // stream schedule: rows per shared-memory tile (kThreads / lanes)
   int tile_bytes[8];        // stream schedule: bytes of a stage's value region (columns follow)
   int max_row;              // nonzeros of the longest row
+  int tile;                 // the vector-load schedule runs from warp tiles where a kernel has them
   int cols_sorted;          // every row's column indices strictly increase
   const double* dinv;       // Jacobi: 1 / a_ii in fp64 when the launch preconditions, else nullptr
   const float* icf;         // IC(0) factor in fp32 when the launch preconditions with it, else
@@ -179,6 +183,7 @@ struct Launch {
   PolicyView pol;
   OptView opt;
   int train;                // 1: epsilon-greedy episode with online private updates
+  int tile;                 // the stepped product kernel has warp tiles (kTileBytes of shared memory)
   int stream_stage;         // bytes of one stage of the stream ring (0: no stream schedule)
   unsigned long long episode;
   double eps;
@@ -248,8 +253,10 @@ constexpr int kPhaseKernels = 6;
 constexpr int kPhaseDone = 10;  // the phase machine's final phase (PH_DONE in solver.cuh)
 cudaError_t stepped_occupancy(int which, int* blocks_per_sm, size_t smem);
 cudaError_t stepped_set_smem_limit(size_t bytes);
+cudaError_t stepped_tile_occupancy(int* blocks_per_sm);  // (sets the tile kernel's limit too)
+cudaError_t spmv_tile_occupancy(int* blocks_per_sm);
 cudaError_t stepped_graph(const Launch& L, const int grids[kPhaseKernels], size_t smem, unsigned limit,
-                          cudaGraph_t* out);
+                          cudaGraph_t* out);  // (kernel 0 with kTileBytes more when L.tile)
 cudaError_t stepped_pass(const Launch& L, const int grids[kPhaseKernels], size_t smem, cudaStream_t s);
 // the IC(0) instantiations (cg_kernel_ic.cu)
 cudaError_t launch_cg_ic(const Launch& L, int grid, size_t smem, cudaStream_t s);
@@ -304,7 +311,8 @@ cudaError_t launch_row_features(int n, const int* rp, const int* ci, const doubl
                                 cudaStream_t s);
 cudaError_t launch_to_format(const double* x, void* xlow, int n, int f, cudaStream_t s);
 cudaError_t launch_from_q(const void* q, const short* rexp, double* y, int n, int f, cudaStream_t s);
-cudaError_t launch_spmv_only(const DevSys& S, int fmt, int grid, int stream_stage, unsigned* err, cudaStream_t s);
+cudaError_t launch_spmv_only(const DevSys& S, int fmt, int grid, int stream_stage, bool tile, unsigned* err,
+                             cudaStream_t s);
 cudaError_t spmv_occupancy(int* blocks_per_sm, size_t smem);
 cudaError_t set_smem_limits(size_t bytes);
 cudaError_t launch_qcopy(const double* Q, double* Qpriv, int nlanes, long long qsize, cudaStream_t s);

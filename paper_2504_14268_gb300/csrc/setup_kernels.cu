@@ -176,6 +176,19 @@ __global__ void __launch_bounds__(kThreads) spmv_standalone(const DevSys S, int 
   spmv_rows(S, Rows{r01[0], r01[1]}, fmt, -1, nu, stream_stage > 0 ? &scx : nullptr);
 }
 
+// The fp64 product from warp tiles, in the shape of the stepped solve's product kernel.
+__global__ void __launch_bounds__(kThreads, 2) spmv_standalone_tile(const DevSys S) {
+  __shared__ int r01[2];
+  extern __shared__ __align__(128) unsigned char dyn[];
+  if (threadIdx.x == 0) {
+    r01[0] = part_row(S.A.rp, S.A.n, S.A.nnz, blockIdx.x, gridDim.x);
+    r01[1] = part_row(S.A.rp, S.A.n, S.A.nnz, blockIdx.x + 1, gridDim.x);
+  }
+  __syncthreads();
+  DotAcc nu{0.0, 0.f, 0.f};
+  spmv_tile(S, Rows{r01[0], r01[1]}, -1, nu, dyn);
+}
+
 // Jacobi preconditioner: dinv[i] = 1 / a_ii in fp64 (one thread per row); a row without a
 // positive diagonal entry sets *bad and gets dinv = 0.
 __global__ void jacobi_diag(int n, const int* __restrict__ rp, const int* __restrict__ ci,
@@ -452,15 +465,26 @@ cudaError_t launch_from_q(const void* q, const short* rexp, double* y, int n, in
   return cudaGetLastError();
 }
 
-cudaError_t launch_spmv_only(const DevSys& S, int fmt, int grid, int stream_stage, unsigned* err, cudaStream_t s) {
+cudaError_t launch_spmv_only(const DevSys& S, int fmt, int grid, int stream_stage, bool tile, unsigned* err,
+                             cudaStream_t s) {
   if (S.A.n == 0) return cudaSuccess;
   cudaGetLastError();
-  spmv_standalone<<<grid, kThreads, stream_stage > 0 ? 2 * (size_t)stream_stage : 0, s>>>(S, fmt, stream_stage, err);
+  if (tile)
+    spmv_standalone_tile<<<grid, kThreads, kTileBytes, s>>>(S);
+  else
+    spmv_standalone<<<grid, kThreads, stream_stage > 0 ? 2 * (size_t)stream_stage : 0, s>>>(S, fmt, stream_stage, err);
   return cudaGetLastError();
 }
 
 cudaError_t spmv_occupancy(int* blocks_per_sm, size_t smem) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, spmv_standalone, kThreads, smem);
+}
+
+cudaError_t spmv_tile_occupancy(int* blocks_per_sm) {
+  const cudaError_t e =
+      cudaFuncSetAttribute(spmv_standalone_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileBytes);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, spmv_standalone_tile, kThreads, kTileBytes);
 }
 
 cudaError_t cg_set_smem_limit(size_t bytes);

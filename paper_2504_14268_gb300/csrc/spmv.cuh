@@ -496,6 +496,83 @@ __device__ void spmv_vload(const DevSys& S, const VT* __restrict__ vals, const V
   long_pass<VT, COMP>(lr, S, vals, xin, p1, nu_fmt, nu);
 }
 
+// One thread per row from warp tiles, fp64: a warp takes 32 consecutive rows, copies their contiguous
+// columns and values to its own part of shared memory with coalesced asynchronous 16-byte copies
+// (no registers in between), and every lane then walks its row there, in column order as
+// spmv_vload does, so the sums are the same bit for bit. What bounds the direct loads of rows of
+// 16 and more nonzeros is the L1: a warp's 16-byte loads fall on 32 different lines, some 700 line
+// look-ups per 32 rows of 27 nonzeros against 150 this way. Two thirds of the gathers miss the L1,
+// so a row takes as many round trips to L2 as it has batches of gathers: the kernels that run this
+// allow 128 registers a thread for batches of 9 (with 4 at 64 registers it was no faster than the
+// direct loads). fp64 27-point products: 100^3 91.0 -> 84.9 us, 140^3 213.5 -> 202.8, 220^3
+// 765 -> 736; 143^3 CG of 60 iterations 19.22 -> 17.35 ms. The other formats stay with the direct
+// loads (this way at 220^3: fp32 484 -> 492 us, tf32 543 -> 612, fp16 454 -> 537).
+// Other warps of the SM compute while a warp's copies are on their way. For matrices no 32
+// consecutive rows of which exceed a tile (DevMatrix::tile); the next tile's row bounds are
+// loaded while this one is summed.
+__device__ __forceinline__ void cp_async16(unsigned dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void spmv_tile(const DevSys& S, Rows R, int nu_fmt, DotAcc& nu, unsigned char* buf) {
+  constexpr int U = 9;  // gathers in flight per lane
+  const double* __restrict__ vals = S.A.v64;
+  const double* xin = S.p;
+  const int* __restrict__ rp = S.A.rp;
+  const int* __restrict__ ci = S.A.ci;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int* sc = reinterpret_cast<int*>(buf + (size_t)w * kTileWarpBytes);
+  double* sv = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(sc) + 4 * (kTileEntries + 8));
+  const unsigned sc32 = smem_u32(sc), sv32 = smem_u32(sv);
+  int base = R.r0 + 32 * w;
+  int ne0 = 0, ne1 = 0;
+  if (base + lane < R.r1) {
+    ne0 = __ldg(rp + base + lane);
+    ne1 = __ldg(rp + base + lane + 1);
+  }
+  for (; base < R.r1; base += kThreads) {
+    const int row = base + lane;
+    const int e0 = ne0, e1 = ne1;
+    const int E0 = __shfl_sync(kFull, e0, 0), E1 = __shfl_sync(kFull, e1, min(31, R.r1 - 1 - base));
+    const int cb = E0 & ~3, vb = E0 & ~1;
+    for (int i = lane; 4 * i < E1 - cb; i += 32) cp_async16(sc32 + 16u * i, ci + cb + 4 * i);
+    for (int i = lane; 2 * i < E1 - vb; i += 32) cp_async16(sv32 + 16u * i, vals + vb + 2 * i);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const double pi = row < R.r1 ? nu_input(S, xin, row, F64, nu_fmt) : 0.0;
+    if (row + kThreads < R.r1) {
+      ne0 = __ldg(rp + row + kThreads);
+      ne1 = __ldg(rp + row + kThreads + 1);
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+    if (row < R.r1) {
+      const int* c = sc + (e0 - cb);
+      const double* v = sv + (e0 - vb);
+      const int len = e1 - e0;
+      RowAcc<double, false> acc;
+      int k = 0;
+      for (; k + U <= len; k += U) {
+        double x[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) x[j] = xin[c[k + j]];
+#pragma unroll
+        for (int j = 0; j < U; ++j) acc.add(v[k + j], x[j]);
+      }
+      if (k < len) {
+        double x[U];
+#pragma unroll
+        for (int j = 0; j < U - 1; ++j)
+          if (k + j < len) x[j] = xin[c[k + j]];
+#pragma unroll
+        for (int j = 0; j < U - 1; ++j)
+          if (k + j < len) acc.add(v[k + j], x[j]);
+      }
+      finish_row<double, false>(S, row, e0, e1, acc, F64, nu_fmt, pi, nu, [&](int k) { return ldg_val(vals + k); },
+                           [&](int k) { return __ldg(ci + k); }, xin);
+    }
+    __syncwarp();  // the tile is read before the next one replaces it
+  }
+}
+
 // Staged stream CSR: the CTA's rows are cut into tiles of kThreads / K rows; the tile's
 // contiguous value and column ranges are fetched into a two-stage shared-memory ring with
 // bulk copies (16-byte aligned by rounding the byte ranges out; the matrix arrays are

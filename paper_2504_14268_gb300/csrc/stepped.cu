@@ -94,6 +94,31 @@ __global__ void __launch_bounds__(kThreads, 4) cg_phase(const Launch L) {
   if (threadIdx.x == 0) atomicExch(L.bars, 0u);
 }
 
+// Phase A of solves whose every product is fp64, from warp tiles (spmv_tile): two CTAs per SM, whose
+// tiles fill its shared memory, with 128 registers a thread for the gathers in flight.
+__global__ void __launch_bounds__(kThreads, 2) cg_phase_tile(const Launch L) {
+  __shared__ Smem sm;
+  extern __shared__ __align__(128) unsigned char dyn[];
+  if (threadIdx.x == 0) {
+    sm.lk_phase = ((const volatile SysState*)L.st)->phase;
+    sm.ok = *(volatile unsigned*)L.err == 0u ? 1 : 0;
+  }
+  __syncthreads();
+  if (sm.lk_phase != PH_A || !sm.ok) return;
+  const DevSys& S = L.sys[0];
+  if (threadIdx.x == 0) {
+    sm.r0 = stepped_row<PH_A>(S, blockIdx.x, gridDim.x);
+    sm.r1 = stepped_row<PH_A>(S, blockIdx.x + 1, gridDim.x);
+  }
+  load_bcast(L.st, sm);  // ends with __syncthreads
+  DotAcc nu{0.0, 0.f, 0.f};
+  spmv_tile(S, Rows{sm.r0, sm.r1}, sm.bc.fmt[2], nu, dyn);
+  lk_partial(L, blockIdx.x, 0, cta_dot(nu, sm.red));
+  if (!arrive_last(L, sm)) return;
+  lk_step_slots<PH_A>(L, 0, 0, gridDim.x, sm);
+  if (threadIdx.x == 0) atomicExch(L.bars, 0u);
+}
+
 // End of a pass through the loop body: continue while the system is not done. bars[16]
 // counts the passes; beyond `limit` the phase machine is taken to be stuck (status word).
 __global__ void cg_loop_ctrl(const Launch L, cudaGraphConditionalHandle h, unsigned limit) {
@@ -107,9 +132,11 @@ __global__ void cg_loop_ctrl(const Launch L, cudaGraphConditionalHandle h, unsig
   if (ph == PH_DONE || err || c >= limit) cudaGraphSetConditional(h, 0u);
 }
 
-const void* phase_kernel(int which) {
+const void* phase_kernel(int which, bool tile = false) {
   switch (which) {
-    case 0: return (const void*)cg_phase<PH_A>;
+    case 0:
+      if (tile) return (const void*)cg_phase_tile;
+      return (const void*)cg_phase<PH_A>;
     case 1: return (const void*)cg_phase<PH_B>;
     case 2: return (const void*)cg_phase<PH_C>;
     case 4: return (const void*)cg_phase<PH_W>;
@@ -118,10 +145,24 @@ const void* phase_kernel(int which) {
   }
 }
 
+// Dynamic shared memory of kernel w: the stream ring, or the product kernel's warp tiles (a launch
+// has one or the other).
+size_t phase_smem(const Launch& L, int w, size_t ring) {
+  if (w == 0 && L.tile) return kTileBytes;
+  return w == 0 || w == 3 || w == 4 ? ring : 0;
+}
+
 }  // namespace
 
 cudaError_t stepped_occupancy(int which, int* blocks_per_sm, size_t smem) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, phase_kernel(which), kThreads, smem);
+}
+
+cudaError_t stepped_tile_occupancy(int* blocks_per_sm) {
+  const cudaError_t e =
+      cudaFuncSetAttribute(cg_phase_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileBytes);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, cg_phase_tile, kThreads, kTileBytes);
 }
 
 cudaError_t stepped_set_smem_limit(size_t bytes) {
@@ -142,8 +183,8 @@ cudaError_t stepped_pass(const Launch& L, const int grids[kPhaseKernels], size_t
   void* args[] = {(void*)&Lc};
   for (int i = 0; i < nbody; ++i) {
     const int w = body_k[i];
-    const cudaError_t e = cudaLaunchKernel(phase_kernel(w), dim3(grids[w]), dim3(kThreads), args,
-                                           (w == 0 || w == 3 || w == 4) ? smem : 0, s);
+    const cudaError_t e = cudaLaunchKernel(phase_kernel(w, L.tile), dim3(grids[w]), dim3(kThreads), args,
+                                           phase_smem(L, w, smem), s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -181,10 +222,10 @@ cudaError_t stepped_graph(const Launch& L, const int grids[6], size_t smem, unsi
     const int w = body_k[i];
     cudaKernelNodeParams kp;
     memset(&kp, 0, sizeof(kp));
-    kp.func = (void*)phase_kernel(w);
+    kp.func = (void*)phase_kernel(w, L.tile);
     kp.gridDim = dim3(grids[w]);
     kp.blockDim = dim3(kThreads);
-    kp.sharedMemBytes = (w == 0 || w == 3 || w == 4) ? (unsigned)smem : 0u;
+    kp.sharedMemBytes = (unsigned)phase_smem(L, w, smem);
     kp.kernelParams = args;
     cudaGraphNode_t nd;
     e = cudaGraphAddKernelNode(&nd, body, prev ? &prev : nullptr, prev ? 1 : 0, &kp);
