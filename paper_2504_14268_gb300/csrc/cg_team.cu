@@ -8,15 +8,13 @@ namespace {
 constexpr size_t kTeamSmemMax = 227 * 1024;
 }
 
-size_t team_fixed_smem() { return kTeamFixed; }
 size_t team_max_heap() { return kTeamSmemMax - kTeamFixed; }
 
 // Sets the kernels' limits; *max_cluster receives the largest cluster that fits the device,
 // resident[i] how many clusters of 2^i CTAs run at a time.
 cudaError_t team_setup(int* max_cluster, int resident[5]) {
   cudaError_t e = cudaFuncSetAttribute(cg_team<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTeamSmemMax);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(cg_team<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTeamSmemMax);
+  if (e == cudaSuccess) e = team_setup_grid(kTeamSmemMax);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(cg_team<true, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e == cudaSuccess) e = team_setup_ic(kTeamSmemMax);
   if (e != cudaSuccess) return e;
@@ -45,11 +43,8 @@ cudaError_t team_setup(int* max_cluster, int resident[5]) {
 }
 
 cudaError_t launch_cg_team(const Launch& L, int cluster, int grid, cudaStream_t s) {
+  if (cluster == 0) return launch_cg_team_grid(L, grid, s);
   const size_t smem = kTeamFixed + (size_t)L.team_heap;
-  if (cluster == 0) {
-    void* args[] = {(void*)&L};
-    return cudaLaunchCooperativeKernel((const void*)cg_team<false, false>, dim3(grid), dim3(kTT), args, smem, s);
-  }
   if (L.ic) return launch_cg_team_ic(L, cluster, grid, smem, s);
   return team_launch_cluster(cg_team<true, false>, L, cluster, grid, smem, s);
 }

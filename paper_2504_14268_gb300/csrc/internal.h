@@ -22,7 +22,11 @@ constexpr int kBarStride = 32;      // uint32 words between team barriers (128 b
 constexpr int kTileEntries = 896;   // nonzeros of a warp's tile (32 rows) of the vector-load schedule
 constexpr int kTileWarpBytes = 4 * (kTileEntries + 8) + 8 * (kTileEntries + 2);  // columns, fp64 values
 constexpr int kTileBytes = kTileWarpBytes * (kThreads / 32);
-constexpr int kTeamThreads = 1024;  // threads per CTA of the team solver
+// Threads per CTA of the team solver: 512 leave 128 registers for loads in flight, and a barrier takes 30
+// to 79 cycles with the warps it holds (against 1024: training on 8 systems 2.48 -> 2.41 ms, IC(0) on a
+// 28^3 27-point system 4.77 -> 4.36, a 160,000-row graph 0.94 -> 0.91).
+constexpr int kTeamThreads = 512;
+constexpr int kTeamTileWarp = 7232; // bytes of a warp's product tile
 constexpr int kTeamIcBars = 32;    // level blocks of the IC(0) substitutions in flight at most
 constexpr int kTeamMaxCluster = 16; // CTAs of a cluster team at most
 constexpr int kStageBytes = 24 * 1024;  // one stage of the stream schedule's shared-memory ring
@@ -272,11 +276,12 @@ cudaError_t cg_occupancy(int* blocks_per_sm, size_t smem);
 size_t cg_static_smem();
 // Team solver (cg_team.cu): clusters of `cluster` CTAs holding the teams of L.team_cta, or 0: `grid`
 // CTAs as one team on system 0 (cooperative launch).
-size_t team_fixed_smem();
 size_t team_max_heap();
 cudaError_t team_setup(int* max_cluster, int resident[5]);
 cudaError_t launch_cg_team(const Launch& L, int cluster, int grid, cudaStream_t s);
 cudaError_t team_setup_ic(size_t smem_max);  // (cg_team_ic.cu)
+cudaError_t team_setup_grid(size_t smem_max);  // (cg_team_grid.cu)
+cudaError_t launch_cg_team_grid(const Launch& L, int grid, cudaStream_t s);
 cudaError_t launch_cg_team_ic(const Launch& L, int cluster, int grid, size_t smem, cudaStream_t s);
 cudaError_t launch_validate(int n, long long nnz, const int* rp, const int* ci, const double* v,
                             unsigned* flags, int* bad_row, cudaStream_t s);

@@ -28,6 +28,7 @@ constexpr int kIcBars = kTeamIcBars;
 constexpr int kTW = kTT / 32;
 constexpr int kXV = 4;            // values per exchange at most
 constexpr int kMidRow = 32;       // longer rows are summed by a warp
+constexpr int kShortRow = 8;      // matrices of rows up to this load a row at once
 constexpr int kLongBatch = 16;    // rows summed by the CTA between two barriers
 constexpr int kLongRowTeam = 512; // ... and longer ones by the CTA (fp32: kLongRow, see team_product)
 
@@ -54,6 +55,7 @@ struct TeamSmem {
   float2 lcorr[kLongBatch][kTW];
   int lrow[kLongBatch];
   int nq, nl;  // queued rows (zero between products)
+  unsigned char* tile;            // the warps' tiles of the product, or nullptr
   const int *rp, *ci;             // the row bounds and columns, the matrix's or the CTA's own copy, ...
   int rbase, ebase;               // ... whose first elements are these rows and entries
   int queue[kTT];
@@ -446,9 +448,71 @@ __device__ __noinline__ void team_queued(TeamSmem& t, const VT* __restrict__ val
   __syncthreads();
 }
 
+// The product from warp tiles (spmv_tile's scheme), the tile being 32 rows of values of up to four
+// bytes; fp64 rows, whose sum has no order to keep, come 16 to a tile with two lanes each. (64^3
+// 27-point system on the whole grid, tf32: 23 us a product from direct loads.)
+template <typename VT, bool COMP>
+__device__ __forceinline__ void team_tiles(TeamSmem& t, const VT* __restrict__ vals, const VT* xin, int p1, double* q) {
+  constexpr int PER = 16 / (int)sizeof(VT);
+  constexpr int LPR = sizeof(VT) == 8 ? 2 : 1;  // lanes per row
+  constexpr int TR = 32 / LPR;
+  constexpr int CAP = sizeof(VT) == 8 ? 592 : 896;
+  constexpr int U = sizeof(VT) == 8 ? 7 : 14;
+  static_assert(4 * (CAP + 8) + (int)sizeof(VT) * (CAP + PER) <= kTeamTileWarp, "a tile exceeds its place");
+  const int* __restrict__ ci = t.S.A.ci;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int* sc = reinterpret_cast<int*>(t.tile + (size_t)w * kTeamTileWarp);
+  VT* sv = reinterpret_cast<VT*>(reinterpret_cast<unsigned char*>(sc) + 4 * (CAP + 8));
+  const unsigned sc32 = smem_u32(sc), sv32 = smem_u32(sv);
+  const int r0 = t.V.r0, r1 = r0 + t.V.n, rb = t.rbase;
+  const int* rp = t.rp;
+  for (int base = r0 + TR * w; base < r1; base += TR * kTW) {
+    const int row = base + lane / LPR;
+    const int e0 = rp[min(row, r1) - rb], e1 = rp[min(row + 1, r1) - rb];
+    const int E0 = __shfl_sync(kFull, e0, 0), E1 = __shfl_sync(kFull, e1, 31);
+    const int cb = E0 & ~3, vb = E0 & ~(PER - 1);
+    const bool staged = E1 - E0 <= CAP;
+    if (staged) {
+      for (int i = lane; 4 * i < E1 - cb; i += 32) cp_async16(sc32 + 16u * i, ci + cb + 4 * i);
+      for (int i = lane; PER * i < E1 - vb; i += 32) cp_async16(sv32 + 16u * i, vals + vb + PER * i);
+      asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+      __syncwarp();
+    }
+    RowAcc<VT, COMP> acc;
+    const int len = e1 - e0, k0 = lane & (LPR - 1);
+    const int* c = staged ? sc + (e0 - cb) : ci + e0;
+    const VT* v = staged ? sv + (e0 - vb) : vals + e0;
+    int k = k0;
+    for (; k + LPR * (U - 1) < len; k += LPR * U) {
+      VT x[U];
+#pragma unroll
+      for (int j = 0; j < U; ++j) x[j] = xin[c[k + LPR * j]];
+#pragma unroll
+      for (int j = 0; j < U; ++j) acc.add(v[k + LPR * j], x[j]);
+    }
+    if (k < len) {
+      VT x[U];
+#pragma unroll
+      for (int j = 0; j < U - 1; ++j)
+        if (k + LPR * j < len) x[j] = xin[c[k + LPR * j]];
+#pragma unroll
+      for (int j = 0; j < U - 1; ++j)
+        if (k + LPR * j < len) acc.add(v[k + LPR * j], x[j]);
+    }
+    if constexpr (LPR == 2) acc.step(kFull, 1);
+    if (row < r1 && k0 == 0) team_finish<VT, COMP>(t, vals, xin, p1, q, row, len, acc);
+    __syncwarp();  // the tile is read before the next one replaces it
+  }
+  if (LPR > 1) __syncthreads();  // rows finished by other threads than their own
+}
+
 template <typename VT, bool COMP>
 __device__ __forceinline__ void team_product(TeamSmem& t, const VT* __restrict__ vals, const VT* xin, int p1, double* q) {
   const DevSys& S = t.S;
+  if (t.tile && S.A.sched[p1] == SCHED_VLOAD) {
+    team_tiles<VT, COMP>(t, vals, xin, p1, q);
+    return;
+  }
   const int* rp = t.rp;  // in shared memory when they fit
   const int* ci = t.ci;
   const int rbase = t.rbase, ebase = t.ebase;
@@ -460,6 +524,7 @@ __device__ __forceinline__ void team_product(TeamSmem& t, const VT* __restrict__
   const int K = vload ? 1 : S.A.lanes[p1];
   const int mid = vload && !kOrdered ? kMidRow : kLong;  // longer rows are queued
   const bool queueing = S.A.max_row > mid;               // the same for the whole team
+  const bool shortrows = vload && S.A.max_row <= kShortRow;
   const int chunk = kTT / K;
   for (int base = r0; base < r1; base += chunk) {
     const int row = base + (int)threadIdx.x / K;
@@ -471,6 +536,25 @@ __device__ __forceinline__ void team_product(TeamSmem& t, const VT* __restrict__
           if (e1 - e0 > kLong) t.queue[kTT - 1 - atomicAdd(&t.nl, 1)] = row;
           else t.queue[atomicAdd(&t.nq, 1)] = row;
         }
+      } else if (sizeof(VT) >= 4 && shortrows) {
+        // all loads of the row at once: from 16-byte groups a row of five doubles is two or three
+        // round trips to L2, one after the other
+        const int len = e1 - e0;
+        const int* c = ci + (e0 - ebase);
+        VT v[kShortRow], x[kShortRow];
+#pragma unroll
+        for (int j = 0; j < kShortRow; ++j)
+          v[j] = x[j] = VT();
+#pragma unroll
+        for (int j = 0; j < kShortRow; ++j)
+          if (j < len) {
+            v[j] = ldg_val(vals + e0 + j);
+            x[j] = xin[c[j]];
+          }
+#pragma unroll
+        for (int j = 0; j < kShortRow; ++j)
+          if (j < len) acc.add(v[j], x[j]);
+        team_finish<VT, COMP>(t, vals, xin, p1, q, row, len, acc);
       } else if (vload) {
         constexpr int G = sizeof(VT) <= 2 ? 8 : 4;
         constexpr int NV = G * (int)sizeof(VT) / 16;
@@ -1230,14 +1314,18 @@ __global__ void __launch_bounds__(kTT, 1) cg_team(const __grid_constant__ Launch
     }
   }
   __syncthreads();
-  // Row bounds and columns to shared memory when there is room: the product's chain of dependent
-  // loads then has one step outside it (the values and the gathers, issued together) instead of three.
+  // The warps' product tiles, then (without tiles) the row bounds and columns to shared memory when
+  // there is room: the product's chain of dependent loads then has one step outside it (the values
+  // and the gathers, issued together) instead of three.
   {
     const int n = t.V.n, r0 = t.V.r0;
     const long long room0 = room - 4LL * n;
+    const bool shared = t.V.r == heap0;
+    double* const after = shared ? heap0 + 4LL * n : heap0;
+    const bool tiles = t.S.A.tile && L.tile && (long long)kTeamTileWarp * kTW / 8 + 2 <= (shared ? room0 : room);
     const int ea = n > 0 ? __ldg(t.S.A.rp + r0) & ~7 : 0, eb = n > 0 ? (__ldg(t.S.A.rp + r0 + n) + 7) & ~7 : 0;
     const long long words = (long long)(eb - ea) + n + 8;
-    const bool fits = t.V.r == heap0 && words / 2 + 2 <= room0;
+    const bool fits = shared && !tiles && words / 2 + 2 <= room0;
     int* cs = reinterpret_cast<int*>(reinterpret_cast<unsigned long long>(heap0 + 4LL * n + 1) & ~15ull);
     int* rs = cs + (eb - ea);
     if (fits) {
@@ -1245,6 +1333,7 @@ __global__ void __launch_bounds__(kTT, 1) cg_team(const __grid_constant__ Launch
       for (int i = threadIdx.x; i <= n && n > 0; i += kTT) rs[i] = __ldg(t.S.A.rp + r0 + i);
     }
     if (threadIdx.x == 0) {
+      t.tile = tiles ? reinterpret_cast<unsigned char*>((reinterpret_cast<unsigned long long>(after + 1)) & ~15ull) : nullptr;
       // (no pointer is moved below its array: shared addresses are 32 bits wide)
       t.rp = fits ? rs : t.S.A.rp;
       t.ci = fits ? cs : t.S.A.ci;
