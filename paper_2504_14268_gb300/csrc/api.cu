@@ -83,7 +83,10 @@ struct Plan {
   bool lockstep = false;
   bool team = false;         // the team solver: one cluster per system, or the whole grid on one
   int team_cluster = 0;      // ... CTAs of a cluster (0: the whole grid)
-  DevBuf xch;                // ... exchange words of the whole-grid team
+  // ... its tables in one upload (systems, the clusters' CTAs) and its small outputs in one block:
+  // exchange words of the whole-grid team, the status word (both zeroed per launch), results
+  DevBuf tin, tout;
+  std::vector<unsigned char> hin, hout;
   size_t xch_bytes = 0;
   bool stepped = false;      // one system, one kernel per phase in a while-loop graph
   bool stepped_host = false; // ... the passes launched by the host instead (option stepped = 3)
@@ -669,13 +672,9 @@ mpcg_status build_team_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& 
       for (int r = 0; r < sz; ++r) c[r] = make_int4(i, r, sz, used);
       used += sz;
     }
-    CK(ctx, pl.cta_team.ensure(sizeof(int4) * ctas.size()));
-    CK(ctx, cudaMemcpyAsync(pl.cta_team.p, ctas.data(), sizeof(int4) * ctas.size(), cudaMemcpyHostToDevice, s));
-    CK(ctx, cudaStreamSynchronize(s));  // (pageable host memory)
   }
   const int grid = cluster ? (int)ctas.size() : ctx->nsm;
   pl.xch_bytes = cluster ? 0 : 2 * 4 * sizeof(uint4) * (size_t)grid;
-  if (pl.xch_bytes) CK(ctx, pl.xch.ensure(pl.xch_bytes));
   // Shared memory: the fixed part, the whole-grid exchange's values, the private table, and the
   // vectors of the largest share of rows (even shares of nnz + 4 n; of rows half as long as the
   // mean, as at grid boundaries, a share holds that many). A CTA whose rows exceed what was given
@@ -710,23 +709,27 @@ mpcg_status build_team_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& 
   }
   heap += (cluster ? 0 : 8 * 4 * (size_t)grid) + 8 * (size_t)(team_q + (team_v + 1) / 2 + 1);
   heap = std::min((heap + 127) / 128 * 128, team_max_heap());
-  CK(ctx, pl.sys.ensure(sizeof(DevSys) * nsys));
   CK(ctx, pl.st.ensure(sizeof(SysState) * nsys));
-  CK(ctx, pl.res.ensure(sizeof(mpcg_result) * nsys));
-  CK(ctx, pl.err.ensure(sizeof(unsigned)));
-  CK(ctx, cudaMemcpyAsync(pl.sys.p, pl.hsys.data(), sizeof(DevSys) * nsys, cudaMemcpyHostToDevice, s));
+  const size_t sys_bytes = (sizeof(DevSys) * nsys + 15) / 16 * 16, cta_bytes = sizeof(int4) * ctas.size();
+  pl.hin.resize(sys_bytes + cta_bytes);
+  memcpy(pl.hin.data(), pl.hsys.data(), sizeof(DevSys) * nsys);
+  if (cta_bytes) memcpy(pl.hin.data() + sys_bytes, ctas.data(), cta_bytes);
+  CK(ctx, pl.tin.ensure(pl.hin.size()));
+  CK(ctx, pl.tout.ensure(pl.xch_bytes + 16 + sizeof(mpcg_result) * nsys));
+  CK(ctx, cudaMemcpyAsync(pl.tin.p, pl.hin.data(), pl.hin.size(), cudaMemcpyHostToDevice, s));
+  unsigned char* out = pl.tout.as<unsigned char>();
   pl.grid = grid;
   pl.nsys = nsys;
   pl.nteams = 0;
   Launch& L = pl.L;
   memset(&L, 0, sizeof(L));
-  L.sys = pl.sys.as<DevSys>();
+  L.sys = pl.tin.as<DevSys>();
   L.st = pl.st.as<SysState>();
   L.nsys = nsys;
-  L.team_cta = pl.cta_team.as<int4>();
-  L.res = pl.res.as<mpcg_result>();
-  L.err = pl.err.as<unsigned>();
-  L.xch = pl.xch.as<uint4>();
+  L.team_cta = reinterpret_cast<const int4*>(pl.tin.as<unsigned char>() + sys_bytes);
+  L.xch = reinterpret_cast<uint4*>(out);
+  L.err = reinterpret_cast<unsigned*>(out + pl.xch_bytes);
+  L.res = reinterpret_cast<mpcg_result*>(out + pl.xch_bytes + 16);
   L.team_heap = (int)heap;
   L.tile = tiles ? 1 : 0;
   L.team_q = team_q;
@@ -968,8 +971,7 @@ mpcg_status build_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& in, m
 // Enqueues one launch of a built plan (barrier counters and status word cleared first).
 mpcg_status enqueue_plan(mpcg_ctx_t ctx, Plan& pl, cudaStream_t s) {
   if (pl.team) {
-    CK(ctx, cudaMemsetAsync(pl.err.p, 0, sizeof(unsigned), s));
-    if (pl.xch_bytes) CK(ctx, cudaMemsetAsync(pl.xch.p, 0, pl.xch_bytes, s));
+    CK(ctx, cudaMemsetAsync(pl.tout.p, 0, pl.xch_bytes + 16, s));
     cudaGetLastError();
     CK(ctx, launch_cg_team(pl.L, pl.team_cluster, pl.grid, s));
     return MPCG_OK;
@@ -1029,13 +1031,21 @@ mpcg_status enqueue_plan(mpcg_ctx_t ctx, Plan& pl, cudaStream_t s) {
 
 mpcg_status finish_plan(mpcg_ctx_t ctx, Plan& pl, mpcg_result* res, cudaStream_t s) {
   unsigned herr = 0;
-  pl.hres.resize(std::max(pl.nsys, 1));
-  if (pl.nsys) CK(ctx, cudaMemcpyAsync(pl.hres.data(), pl.res.p, sizeof(mpcg_result) * pl.nsys, cudaMemcpyDeviceToHost, s));
-  CK(ctx, cudaMemcpyAsync(&herr, pl.err.p, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
   unsigned passes = 0;  // the stepped graph's pass counter (bars[16], kept by its control kernel)
-  if (pl.stepped && !pl.stepped_host)
-    CK(ctx, cudaMemcpyAsync(&passes, pl.bars.as<unsigned>() + 16, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-  CK(ctx, cudaStreamSynchronize(s));
+  pl.hres.resize(std::max(pl.nsys, 1));
+  if (pl.team) {  // status word and results in one copy
+    pl.hout.resize(16 + sizeof(mpcg_result) * pl.nsys);
+    CK(ctx, cudaMemcpyAsync(pl.hout.data(), pl.L.err, pl.hout.size(), cudaMemcpyDeviceToHost, s));
+    CK(ctx, cudaStreamSynchronize(s));
+    memcpy(&herr, pl.hout.data(), sizeof(herr));
+    memcpy(pl.hres.data(), pl.hout.data() + 16, sizeof(mpcg_result) * pl.nsys);
+  } else {
+    if (pl.nsys) CK(ctx, cudaMemcpyAsync(pl.hres.data(), pl.res.p, sizeof(mpcg_result) * pl.nsys, cudaMemcpyDeviceToHost, s));
+    CK(ctx, cudaMemcpyAsync(&herr, pl.err.p, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+    if (pl.stepped && !pl.stepped_host)
+      CK(ctx, cudaMemcpyAsync(&passes, pl.bars.as<unsigned>() + 16, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+    CK(ctx, cudaStreamSynchronize(s));
+  }
   if (herr == DERR_TIMEOUT) return fail(ctx, MPCG_ERR_TIMEOUT, "a device-side barrier wait exceeded its limit");
   if (herr) return fail(ctx, MPCG_ERR_INTERNAL, "device status word %u", herr);
   int launches = 1;
