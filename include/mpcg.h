@@ -122,9 +122,10 @@ typedef struct {
                               recompute r = b - A x in fp64, restart with p = r and finish
                               with every operation in fp64 (at most once per solve)     */
   int32_t mlp_hidden;      /* hidden width of the MLP policy (64)                       */
-  int32_t batch_mode;      /* launches with several systems: 0 = automatic (lockstep),
-                            * 1 = teams (each system solved by its own group of CTAs from
-                            * start to end), 2 = lockstep (every CTA works on a slice of
+  int32_t batch_mode;      /* launches with several systems: 0 = automatic (teams when all of
+                            * them run at a time and are estimated to end sooner, else
+                            * lockstep), 1 = teams (each system solved by its own group of
+                            * CTAs from start to end), 2 = lockstep (every CTA works on a slice of
                             * every unfinished system at every phase; slices re-cut as
                             * systems finish)                                            */
   int32_t precond;         /* 0: M = I (op 2 is z = fl_p2(r)); 1: Jacobi, M = diag(A): op 2
@@ -144,14 +145,14 @@ typedef struct {
                             * mpcg_result.near_edge_count: there a rounding-level change of
                             * rho can move the state to the next bin (5e-3)              */
   int32_t stepped;         /* single solves (mpcg_solve): 0 = automatic (stepped for systems
-                            * of at least 2^24 nonzeros without IC(0)), 1 = one persistent
-                            * cooperative launch, 2 = stepped: one kernel per phase of the
+                            * of at least 2^24 nonzeros without IC(0)), 1 = one launch of
+                            * a team (a cluster or the whole grid), 2 = stepped: one kernel per phase of the
                             * iteration, repeated on the device by a conditional while-loop
                             * CUDA graph, 3 = the same kernels with each pass launched by the
                             * host, which reads the phase back after every pass (for tools
                             * that cannot follow kernels inside graphs with conditional
-                            * nodes; slower) (precond = 2 always runs the persistent launch,
-                            * whose substitutions need every CTA resident)              */
+                            * nodes; slower) (precond = 2 always runs as one launch, whose
+                            * substitutions need every CTA resident)                    */
   int32_t variant;         /* 0: the CG of Section 3 (three reductions per iteration); 1: the
                             * single-reduction iteration of Chronopoulos and Gear (an
                             * extension, equal to CG in exact arithmetic): u = fl_p2(M^-1 r),
@@ -185,7 +186,7 @@ typedef struct {
   int32_t near_edge_count; /* greedy tabular decisions taken within edge_tol of a residual-bin
                               edge (options.edge_tol); 0 for other policies             */
   int32_t kernel_launches; /* the library's solver-kernel launches of the call: 1 for one
-                              persistent or lockstep launch (shared by a batch), passes x
+                              team, persistent or lockstep launch (shared by a batch), passes x
                               kernels for the stepped solve (the phase kernels and the loop
                               control kernel of every pass of the graph)               */
 } mpcg_result;
@@ -335,16 +336,17 @@ mpcg_status mpcg_policy_destroy(mpcg_policy_t P);
 
 /* Solves A x = b with the policy (Algorithm 2 for QTABLE/MLP policies) until
  * ||r_{k+1}|| / ||b|| < tol with k >= min_k, max_iter iterations, or breakdown
- * (non-positive or non-finite p^T A p, non-finite residual). One cooperative launch of the
- * persistent kernel runs every iteration on the device. b and x: n doubles, host or device.
+ * (non-positive or non-finite p^T A p, non-finite residual). Every iteration runs on
+ * the device, in one launch of a team or (options.stepped) as a graph of phase kernels.
+ * b and x: n doubles, host or device.
  * history (optional): device or host array of history_cap records. Synchronises `stream`.
  * Errors: INVALID_ARG, BAD_POLICY, CUDA, OOM, TIMEOUT. */
 mpcg_status mpcg_solve(mpcg_ctx_t ctx, mpcg_matrix_t A, const double* b, double* x, double tol,
                        int32_t max_iter, mpcg_policy_t policy, mpcg_result* res,
                        mpcg_iter_record* history, int32_t history_cap, void* stream);
 
-/* Solves nsys independent systems in one persistent launch: the systems are assigned
- * longest-first to teams of CTAs sized by their nonzeros. b[i], x[i]: device pointers.
+/* Solves nsys independent systems in one launch (options.batch_mode): teams of CTAs sized by
+ * the systems' nonzeros, or all systems in lockstep. b[i], x[i]: device pointers.
  * tol and max_iter: per system (host arrays). res: host array of nsys results.
  * Synchronises `stream`. */
 mpcg_status mpcg_solve_batched(mpcg_ctx_t ctx, int32_t nsys, const mpcg_matrix_t* A,
