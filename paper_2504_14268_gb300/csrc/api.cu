@@ -63,7 +63,7 @@ constexpr size_t kTeamIndexHeap = 112 * 1024;      // shared memory up to which 
 constexpr int kTeamIcRows = 32768;                 // IC(0) in a team: rows of the vector in shared memory
 constexpr size_t kTeamIcRing = 96 * 1024;          // ... bytes of its ring of level blocks at most
 constexpr size_t kTeamIcShared = 180 * 1024;       // ... and of both together
-constexpr long long kTeamQBytes = 48 * 1024;        // largest private Q-table of the team solver
+constexpr long long kTeamQBytes = 48 * 1024;        // largest Q-table the team solver copies to shared memory
 constexpr long long kTuneMinNnz = 4LL << 20;        // smallest matrix the autotuner times
 
 }  // namespace
@@ -594,16 +594,16 @@ TeamEstimate team_sizes(mpcg_ctx_t ctx, const std::vector<SysIn>& in, int most, 
 }
 
 // The team solver takes a launch when every product of its matrices runs one of the two
-// row-length schedules, the options are those it implements, and (training) the private table
-// fits beside the vectors. Returns the CTAs per cluster, 0 for the whole grid on one system, -1
-// when another kernel takes the launch.
+// row-length schedules and the options are those it implements. Returns the CTAs per cluster, 0
+// for the whole grid on one system, -1 when another kernel takes the launch. Training rounds and the
+// collection of transitions stay with the other kernels: the team's sums run in another order, an
+// iteration in low formats multiplies a last-bit difference of the residual (a table of eight 16^3 to
+// 30^3 27-point systems moved by 8e-9, single entries by 2e-7), and a learner that meets near-equal
+// actions keeps one or the other by it; there a seed gives the same table as ever.
 int team_rule(mpcg_ctx_t ctx, const std::vector<SysIn>& in, mpcg_policy_t policy, int train) {
   const int nsys = (int)in.size();
-  if (nsys < 1 || ctx->max_cluster < 1 || ctx->opt.variant != 0 || ctx->opt.batch_mode == 2) return -1;
+  if (nsys < 1 || train || ctx->max_cluster < 1 || ctx->opt.variant != 0 || ctx->opt.batch_mode == 2) return -1;
   const bool ic = ctx->opt.precond == 2;
-  // Training with IC(0) stays with the lockstep kernel: a learner that meets near-equal actions keeps
-  // one or the other by the last bits of the residual, and there a seed gives the same table as ever.
-  if (train && ic) return -1;
   const int S = ctx->opt.b_bins * ctx->opt.r_bins, joint = ctx->opt.joint ? 1 : 0;
   const size_t table = policy->kind == 2 ? (size_t)kTeamQBytes + 4 * (size_t)visits_size(S, joint) : 0;
   for (const SysIn& s : in) {  // the ring, the vector and the table fit a CTA's shared memory
@@ -613,7 +613,6 @@ int team_rule(mpcg_ctx_t ctx, const std::vector<SysIn>& in, mpcg_policy_t policy
   for (const SysIn& s : in)
     for (int f = 0; f < NFMT; ++f)
       if (s.A->dm.sched[f] != SCHED_VLOAD && s.A->dm.sched[f] != SCHED_VECTOR) return -1;
-  if (train && policy->kind == 2 && 8 * qtable_size(S, ctx->opt.nprec, joint) > kTeamQBytes) return -1;
   if (nsys > 1) {
     // teams when all run at a time (a cluster's places stay taken until its last team is done) and
     // by the estimate below sooner than the lockstep kernel: per CTA 0.84 ns a unit of cost and 10 us
@@ -643,8 +642,8 @@ int team_rule(mpcg_ctx_t ctx, const std::vector<SysIn>& in, mpcg_policy_t policy
 }
 
 // Device tables of a launch of the team solver (systems as in build_plan).
-mpcg_status build_team_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& in, mpcg_policy_t policy, int train,
-                            int trans_cap, int cluster, cudaStream_t s) {
+mpcg_status build_team_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& in, mpcg_policy_t policy, int cluster,
+                            cudaStream_t s) {
   const int nsys = (int)in.size();
   pl.team = true;
   pl.lockstep = pl.stepped = pl.stepped_host = false;
@@ -675,7 +674,7 @@ mpcg_status build_team_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& 
   }
   const int grid = cluster ? (int)ctas.size() : ctx->nsm;
   pl.xch_bytes = cluster ? 0 : 2 * 4 * sizeof(uint4) * (size_t)grid;
-  // Shared memory: the fixed part, the whole-grid exchange's values, the private table, and the
+  // Shared memory: the fixed part, the whole-grid exchange's values, the copy of the table, and the
   // vectors of the largest share of rows (even shares of nnz + 4 n; of rows half as long as the
   // mean, as at grid boundaries, a share holds that many). A CTA whose rows exceed what was given
   // keeps its vectors in global memory.
@@ -737,7 +736,6 @@ mpcg_status build_team_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& 
   const mpcg_status st = fill_policy(ctx, policy, L.pol);
   if (st != MPCG_OK) return st;
   L.opt = ctx->ov;
-  L.train = train;
   L.ic = ctx->opt.precond == 2 ? 1 : 0;
   L.timeout_cycles = kTimeoutCycles;
   if (const char* t = getenv("MPCG_TIMEOUT_CYCLES")) L.timeout_cycles = atoll(t);
@@ -835,7 +833,7 @@ mpcg_status build_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& in, m
   pl.team = false;
   if (!stepped && force_team == 0) {
     const int cluster = team_rule(ctx, in, policy, train);
-    if (cluster >= 0) return build_team_plan(ctx, pl, in, policy, train, trans_cap, cluster, s);
+    if (cluster >= 0) return build_team_plan(ctx, pl, in, policy, cluster, s);
   }
   bool stream_shape = false;
   for (int i = 0; i < nsys; ++i) stream_shape = stream_shape || uses_stream(in[i].A->dm);

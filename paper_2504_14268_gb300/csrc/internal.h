@@ -95,8 +95,8 @@ struct DevSys {
   mpcg_iter_record* hist;   // device array or nullptr
   int hist_cap;
   int pad1;
-  double* Qpriv;            // training: lane-private copy of the tables (team solver: the table in
-                            // shared memory, in inference too)
+  double* Qpriv;            // training: lane-private copy of the tables; team solver (inference): the
+                            // table in shared memory
   const int* vtab;          // team solver: the table's visit counts in shared memory, or nullptr
   Transition* trans;        // training: transitions of this lane's episode
   int trans_cap;

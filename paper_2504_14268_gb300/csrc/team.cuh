@@ -5,7 +5,7 @@
 // cg_persistent pays for each of the three team steps an arrival counter, a reduction by the
 // last CTA, a scalar step on state in global memory and a release that the others poll, about
 // 10 us each. Here
-//   * every CTA keeps its own copy of the system's state, descriptor and (in training) Q-table
+//   * every CTA keeps its own copy of the system's state, descriptor and Q-table
 //     in shared memory and runs the scalar step itself on the same sums in the same order, so
 //     the copies stay equal bit for bit and nothing has to be broadcast;
 //   * a step's partial sums go from each CTA to every other in one message that carries data
@@ -897,7 +897,7 @@ __device__ __forceinline__ void team_store_x(const TeamSmem& t) {
 //
 // One warp's straight-line code runs at about five cycles an instruction here (it is fetched
 // anew every iteration), an fp64 division takes 560 cycles, a square root 600, a comparison 64.
-// The full steps (step_A, step_B: records, training, stopping, breakdowns, features, any policy)
+// The full steps (step_A, step_B: records, stopping, breakdowns, features, any policy)
 // took 1,300 and 6,800 cycles of an iteration; an ordinary iteration of an inference solve needs
 // of them alpha, beta, the residual bin and the four formats. These come here from one warp: the bin
 // and the stopping test by comparing ||r||^2 with the squared thresholds as integers, rho itself
@@ -927,7 +927,7 @@ __device__ __forceinline__ void team_fast_setup(const Launch& L, TeamSmem& t) {
   const double e = thr * t.st.bnorm;
   t.thr2[m] = __double_as_longlong(e * e);
   if (m == 0) {
-    t.fast = !L.train && !t.S.hist && !t.S.feat_log && o.true_every <= 0 &&
+    t.fast = !t.S.hist && o.true_every <= 0 &&
              (L.pol.kind <= 1 || (L.pol.kind == 2 && !o.joint)) && o.edge_tol < 0.1;
     // 2^21 units in the last place: far more than the squares' rounding; with a table also the
     // neighbourhood of an edge that near_edge_count counts
@@ -1255,11 +1255,10 @@ __global__ void __launch_bounds__(kTT, 1) cg_team(const __grid_constant__ Launch
     heap += used;
     room -= used;
   }
-  if (L.team_q) {  // the table: private in training, a copy otherwise (its reads are on the chain)
-    const double* src = L.train ? t.S.Qpriv : L.pol.Q;
-    for (int i = threadIdx.x; i < L.team_q; i += kTT) heap[i] = src[i];
+  if (L.team_q) {  // a copy of the table (its reads are on the chain)
+    for (int i = threadIdx.x; i < L.team_q; i += kTT) heap[i] = L.pol.Q[i];
     int* vis = (int*)(heap + L.team_q);
-    const int nv = !L.train && L.pol.visits ? L.team_v : 0;
+    const int nv = L.pol.visits ? L.team_v : 0;
     for (int i = threadIdx.x; i < nv; i += kTT) vis[i] = L.pol.visits[i];
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1287,11 +1286,7 @@ __global__ void __launch_bounds__(kTT, 1) cg_team(const __grid_constant__ Launch
     if (threadIdx.x == 0) {
       t.sm.r0 = a;
       t.sm.r1 = b;
-      if (t.rank != 0) {  // one CTA of the team writes the records
-        t.S.hist = nullptr;
-        t.S.trans = nullptr;
-        t.S.feat_log = nullptr;
-      }
+      if (t.rank != 0) t.S.hist = nullptr;  // one CTA of the team writes the records
     }
   }
   double* const heap0 = heap;
