@@ -15,6 +15,7 @@
 #include <tuple>
 #include <vector>
 
+#include "ic_ring.h"
 #include "internal.h"
 
 using namespace mpcg;
@@ -446,7 +447,7 @@ mpcg_status ensure_ic0(mpcg_ctx_t ctx, mpcg_matrix_s* M, cudaStream_t s) {
   // levels are even enough not to be blown up by the padding.
   std::vector<float> hF;
   std::vector<unsigned char> blob;
-  std::vector<int4> desc;
+  std::vector<IcBlock> desc;
   size_t block_max = 0, groups_max = 0;
   bool packed = n > 0 && n <= kTeamIcRows;
   if (packed) {
@@ -473,7 +474,7 @@ mpcg_status ensure_ic0(mpcg_ctx_t ctx, mpcg_matrix_s* M, cudaStream_t s) {
         return;
       }
       const size_t at = blob.size();
-      desc.push_back(make_int4((int)(at / 16), (int)(bytes / 16), 0, 0));
+      desc.push_back(IcBlock{(int)(at / 16), (int)(bytes / 16), 0, 0});
       blob.resize(at + bytes, 0);
       unsigned char* o = blob.data() + at;
       ((int*)o)[0] = ng;
@@ -521,29 +522,19 @@ mpcg_status ensure_ic0(mpcg_ctx_t ctx, mpcg_matrix_s* M, cudaStream_t s) {
   ls = sort_by_level(depth, M->icpb, M->icob, M->icwb, M->nlevb);
   if (ls != MPCG_OK) return ls;
   if (packed) pack_levels(depth, false);
-  if (packed) {
-    // places in the ring, in order from its start; a block that would cross the end goes back to the
-    // start. Block l may be written when every earlier block in its way has been consumed, and at
-    // most kTeamIcBars blocks are in flight.
-    const size_t fit = kTeamIcShared / 16 * 16 - 8 * (((size_t)n + 2) / 2);  // beside the vector
-    const int cap = (int)(std::min(std::min(kTeamIcRing, fit) & ~(size_t)15, blob.size()) / 16);
-    int at = 0;
-    for (size_t l = 0; l < desc.size(); ++l) {
-      if (at + desc[l].y > cap) at = 0;
-      desc[l].z = at;
-      at += desc[l].y;
-      int need = std::max(0, (int)l - kTeamIcBars + 1);
-      for (int j = (int)l - 1; j >= need; --j)
-        if (desc[j].z < desc[l].z + desc[l].y && desc[l].z < desc[j].z + desc[j].y) need = j + 1;
-      desc[l].w = need;
-    }
+  // The ring beside the vector; from some 21,500 rows it is smaller than kTeamIcRing, and systems with
+  // wide levels (27-point grids from 30^3, 7-point from 31^3) no longer fit it: other kernels take those.
+  const size_t fit = kTeamIcShared / 16 * 16 - 8 * (((size_t)n + 2) / 2);
+  const int cap = packed ? (int)(std::min(std::min(kTeamIcRing, fit) & ~(size_t)15, blob.size()) / 16) : 0;
+  if (packed && ic_ring_places(desc, cap, kTeamIcBars)) {
     for (size_t l = 0; l + 1 < desc.size(); ++l)  // each block names the next one's place
-      memcpy(blob.data() + (size_t)desc[l].x * 16 + 8, &desc[l + 1].z, 4);
+      memcpy(blob.data() + (size_t)desc[l].from * 16 + 8, &desc[l + 1].at, 4);
+    static_assert(sizeof(IcBlock) == sizeof(int4), "the kernel reads blocks as int4");
     M->icring = cap * 16;
     CK(ctx, M->icblob.ensure(blob.size()));
-    CK(ctx, M->icdesc.ensure(sizeof(int4) * desc.size()));
+    CK(ctx, M->icdesc.ensure(sizeof(IcBlock) * desc.size()));
     CK(ctx, cudaMemcpy(M->icblob.p, blob.data(), blob.size(), cudaMemcpyHostToDevice));
-    CK(ctx, cudaMemcpy(M->icdesc.p, desc.data(), sizeof(int4) * desc.size(), cudaMemcpyHostToDevice));
+    CK(ctx, cudaMemcpy(M->icdesc.p, desc.data(), sizeof(IcBlock) * desc.size(), cudaMemcpyHostToDevice));
     M->icwarps = (int)std::min<size_t>(groups_max, kTeamThreads / 32 - 2);  // (one warp waits, one copies)
     M->bytes += (long long)blob.size();
   }
