@@ -1876,6 +1876,8 @@ mpcg_status mpcg_graph_create(mpcg_ctx_t ctx, int32_t nsys, const mpcg_matrix_t*
   g->plan.reset(new Plan());
   st = build_plan(ctx, *g->plan, in, policy, 0, 0, 0, s);
   if (st != MPCG_OK) return st;
+  // the plan's tables are on their way on s, and a launch may come on any stream
+  CK(ctx, cudaStreamSynchronize(s));
   cudaStream_t cs;
   CK(ctx, cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
   cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
