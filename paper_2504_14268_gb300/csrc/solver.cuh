@@ -211,8 +211,10 @@ __device__ __forceinline__ int state_of(const OptView& o, int k, double rho) {
   int i = k / o.t_width;
   if (i > o.b_bins - 1) i = o.b_bins - 1;
   int j = 0;
-  // non-negative values order as their bit patterns (an fp64 comparison takes 64 cycles)
-  const long long rb = __double_as_longlong(rho);
+  // non-negative values order as their bit patterns (an fp64 comparison takes 64 cycles); a NaN, whose
+  // sign bit may be set, lies above every threshold
+  long long rb = __double_as_longlong(rho);
+  if ((rb & 0x7fffffffffffffffll) > 0x7ff0000000000000ll) rb = 0x7fffffffffffffffll;
   for (int m = 1; m < o.r_bins; ++m) j += (rb <= __double_as_longlong(o.thr[m])) ? 1 : 0;
   return i * o.r_bins + j;
 }
