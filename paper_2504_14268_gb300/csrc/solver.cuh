@@ -220,12 +220,15 @@ __device__ __forceinline__ int state_of(const OptView& o, int k, double rho) {
 }
 
 // 1 when rho lies within edge_tol (relative) of a residual-bin threshold. The fp64 division (some
-// 600 cycles) is made only for thresholds that an fp32 quotient leaves in question.
+// 600 cycles) is made only for thresholds that an fp32 quotient leaves in question, or that are too
+// small for one.
 __device__ __forceinline__ int near_bin_edge(const OptView& o, double rho) {
   int near = 0;
   const float r = (float)rho, lim = (float)o.edge_tol * 1.001f + 1e-5f;
   for (int m = 1; m < o.r_bins; ++m)
-    if (fabsf(__fdividef(r, (float)o.thr[m]) - 1.f) <= lim) near |= fabs(rho / o.thr[m] - 1.0) <= o.edge_tol ? 1 : 0;
+    if (fabsf(__fdividef(r, (float)o.thr[m]) - 1.f) <= lim ||
+        __double_as_longlong(o.thr[m]) < __double_as_longlong(1e-36))
+      near |= fabs(rho / o.thr[m] - 1.0) <= o.edge_tol ? 1 : 0;
   return near;
 }
 
