@@ -72,9 +72,12 @@ __device__ __forceinline__ void load_weights(float* dst, const float* __restrict
   for (int i = threadIdx.x; i < (int)s.np; i += kMlpThreads) dst[i] = __ldg(w + i);
 }
 
-// y_i = act(b_i + sum_j W[i][j] x_j) over j in order, for rows i of n (x: m rows of 32 samples).
+// y_i = act(b_i + sum_j W[i][j] x_j) over j in order, for rows i of n (x: m rows of 32 samples), and 0
+// for lanes without a sample: they then pass nothing back and add nothing to a gradient, even where a
+// weight is not finite.
 template <bool RELU>
-__device__ __forceinline__ void layer(const float* W, const float* b, int n, int m, const float* x, float* y) {
+__device__ __forceinline__ void layer(const float* W, const float* b, int n, int m, const float* x, float* y,
+                                      int samples) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int i0 = w * kNeurons; i0 < n; i0 += kMlpThreads / 32 * kNeurons) {
     const int cnt = min(kNeurons, n - i0);
@@ -90,7 +93,7 @@ __device__ __forceinline__ void layer(const float* W, const float* b, int n, int
     }
 #pragma unroll
     for (int u = 0; u < kNeurons; ++u)
-      if (u < cnt) y[(i0 + u) * kRow + lane] = RELU ? (a[u] > 0.f ? a[u] : 0.f) : a[u];
+      if (u < cnt) y[(i0 + u) * kRow + lane] = lane < samples && (!RELU || a[u] > 0.f) ? a[u] : 0.f;
   }
   __syncthreads();
 }
@@ -162,11 +165,11 @@ __device__ __forceinline__ void layer_grad(const float* dy, int n, const float* 
   }
 }
 
-// The network on the 32 samples in t.f (t.w: its weights): t.h1, t.h2, t.out.
-__device__ __forceinline__ void net(const MlpTile& t, const MlpShape& s) {
-  layer<true>(t.w + s.oW1, t.w + s.ob1, s.H, kNFeat, t.f, t.h1);
-  layer<true>(t.w + s.oW2, t.w + s.ob2, s.H, s.H, t.h1, t.h2);
-  layer<false>(t.w + s.oW3, t.w + s.ob3, s.nout, s.H, t.h2, t.out);
+// The network on the `samples` samples in t.f (t.w: its weights): t.h1, t.h2, t.out.
+__device__ __forceinline__ void net(const MlpTile& t, const MlpShape& s, int samples) {
+  layer<true>(t.w + s.oW1, t.w + s.ob1, s.H, kNFeat, t.f, t.h1, samples);
+  layer<true>(t.w + s.oW2, t.w + s.ob2, s.H, s.H, t.h1, t.h2, samples);
+  layer<false>(t.w + s.oW3, t.w + s.ob3, s.nout, s.H, t.h2, t.out, samples);
 }
 
 // The features of the CTA's samples (row src of `feats` for lane t; zeros for lanes without one).
@@ -204,7 +207,7 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_targets_kernel(const float* _
     if (threadIdx.x < 32) src[threadIdx.x] = b0 + threadIdx.x;
     __syncthreads();
     load_feats(t.f, feats_next, src, cnt);
-    net(t, s);
+    net(t, s, cnt);
     const int smp = threadIdx.x >> 2, j = threadIdx.x & 3;
     if (smp < cnt) y[(b0 + smp) * 4 + j] = target_of(t.out + smp, nprec, j, mask, rew[b0 + smp], done[b0 + smp], gamma);
     __syncthreads();
@@ -247,13 +250,13 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_grad_kernel(
   } else {
     load_weights(t.w, wt, s);
     load_feats(t.f, feats_next, src, cnt);
-    net(t, s);
+    net(t, s, cnt);
     if (smp < cnt) yt[smp][op] = target_of(t.out + smp, nprec, op, mask, rew[src[smp]], done[src[smp]], gamma);
     __syncthreads();
   }
   load_weights(t.w, w, s);
   load_feats(t.f, feats, src, cnt);
-  net(t, s);
+  net(t, s, cnt);
   // output error: only the taken action of each operation carries gradient
   for (int e = threadIdx.x; e < s.nout * 32; e += kMlpThreads) t.dout[(e >> 5) * kRow + (e & 31)] = 0.f;
   __syncthreads();
