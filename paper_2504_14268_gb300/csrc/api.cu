@@ -609,7 +609,11 @@ int team_rule(mpcg_ctx_t ctx, const std::vector<SysIn>& in, mpcg_policy_t policy
     // by the estimate below sooner than the lockstep kernel: per CTA 0.84 ns a unit of cost and 10 us
     // an iteration, against 100 us an iteration and the matrices at 4 TB/s (48 systems of 1,000 to
     // 60,000 rows, 60 iterations: 5.6 against 7.6 ms; 512 systems of 6e8 nonzeros, 5,000
-    // iterations: 71 against 10.7 s). IC(0) substitutions run in the team whenever they can.
+    // iterations: 71 against 10.7 s). IC(0) substitutions run in the team whenever they can. Against the
+    // persistent teams (batch_mode 1), which share the whole grid among a few systems: 85 us an iteration
+    // and the matrices at 5 TB/s, the team's figure without its margin (30 iterations of 27-point fp64 CG:
+    // two 64^3 systems 17.0 ms in clusters of 16, 3.5 ms in persistent teams; eight of 30^3 2.3 against
+    // 3.0; sixteen of 30^3 6.6 against 3.3; two 400^2 five-point systems 2.1 against 2.8).
     const int c8 = std::min(kTeamBatchCluster, ctx->max_cluster);
     int cluster = c8;
     TeamEstimate e = team_sizes(ctx, in, c8, nullptr);
@@ -619,14 +623,15 @@ int team_rule(mpcg_ctx_t ctx, const std::vector<SysIn>& in, mpcg_policy_t policy
       cluster = ctx->max_cluster;
     }
     if (ic) return cluster;
-    if (ctx->opt.batch_mode == 1) return e.one_wave ? cluster : -1;
     double iters = 0, total = 0;
     for (const SysIn& s : in) {
       iters = std::max(iters, (double)s.max_iter);
       total += (double)s.max_iter * (s.A->dm.nnz + 4.0 * s.A->dm.n);
     }
-    const double team = 1.2 * 0.84e-9 * e.time + 10e-6 * iters, lockstep = 100e-6 * iters + 12.0 * total / 4e12;
-    return e.one_wave && team < lockstep ? cluster : -1;
+    const bool teams = ctx->opt.batch_mode == 1;
+    const double team = (teams ? 1.0 : 1.2) * 0.84e-9 * e.time + 10e-6 * iters;
+    const double other = teams ? 85e-6 * iters + 12.0 * total / 5e12 : 100e-6 * iters + 12.0 * total / 4e12;
+    return e.one_wave && team < other ? cluster : -1;
   }
   const long long w = in[0].A->dm.nnz + 4LL * in[0].A->dm.n;
   return ic || w < kTeamGridWork ? ctx->max_cluster : 0;
