@@ -59,7 +59,11 @@ constexpr long long kTimeoutCycles = 4000000000ll;  // about two seconds at 2 GH
 constexpr double kTileMinMean = 14.0;              // mean row length from which warp tiles pay
 constexpr int kTeamBatchCluster = 8;               // cluster of a batch's teams
 constexpr long long kTeamCtaWork = 8192;           // a team has a CTA per so much work (nnz + 4 n)
-constexpr long long kTeamGridWork = 160 * 1000;    // from here a single system takes the whole grid
+constexpr long long kTeamGridWork = 160 * 1000;    // from here a single system takes the whole grid ...
+constexpr int kTeamGridRows = 1200 * 1000;         // ... up to so many rows,
+constexpr int kTeamGridRowsPlain = 1400 * 1000;    // ... with fp64 or fp32 products only up to so many,
+constexpr long long kTeamGridNnz = 1LL << 24;      // ... and below so many nonzeros
+constexpr long long kTeamGridTileNnz = 13 * 1000 * 1000;  // ... fp64 products of a matrix for tiles: up to here
 constexpr size_t kTeamIndexHeap = 112 * 1024;      // shared memory up to which a team's columns are copied
 constexpr int kTeamIcRows = 32768;                 // IC(0) in a team: rows of the vector in shared memory
 constexpr size_t kTeamIcRing = 96 * 1024;          // ... bytes of its ring of level blocks at most
@@ -633,8 +637,22 @@ int team_rule(mpcg_ctx_t ctx, const std::vector<SysIn>& in, mpcg_policy_t policy
     const double other = teams ? 85e-6 * iters + 12.0 * total / 5e12 : 100e-6 * iters + 12.0 * total / 4e12;
     return e.one_wave && team < other ? cluster : -1;
   }
-  const long long w = in[0].A->dm.nnz + 4LL * in[0].A->dm.n;
-  return ic || w < kTeamGridWork ? ctx->max_cluster : 0;
+  // One system: a cluster, from kTeamGridWork on the whole grid (60 iterations: 150^2 five-point 0.84 ms
+  // either way, 180^2 0.84 on the grid, 1.06 in a cluster, 110^2 0.81 and 0.68; 27-point 16^3 0.98 and
+  // 0.68, 24^3 0.97 and 1.31). The grid keeps its lead over the persistent kernel's four CTAs per SM while
+  // the vectors stay in shared memory, up to some 1.05e6 rows, and loses it beyond (30 iterations, fp64 and
+  // tf32, persistent kernel first: five-point 1e6 rows 3.2 / 1.5 and 3.4 / 2.4 ms, 1.2e6 3.2 / 2.7 and
+  // 3.5 / 3.8, 1.44e6 3.4 / 3.1 and 3.7 / 4.5, 2e6 3.9 / 4.1 and 4.3 / 6.2; fp32 1.44e6 3.2 / 2.9; 27-point
+  // 128^3 9.1 / 15.8). An fp64 product without tiles, for
+  // which 27-point systems from 80^3 leave no room, loses it by a little (78^3, with tiles, 3.7 / 2.5 ms,
+  // 80^3 3.7 / 3.8, 84^3 3.9 / 4.3; tf32 3.5 / 3.5, fp32 3.3 / 3.0).
+  const DevMatrix& d = in[0].A->dm;
+  if (ic || d.nnz + 4LL * d.n < kTeamGridWork) return ctx->max_cluster;
+  const bool plain = policy->kind == 0 && (policy->fixed[0] == F64 || policy->fixed[0] == F32);
+  if (d.n > (plain ? kTeamGridRowsPlain : kTeamGridRows) || d.nnz >= kTeamGridNnz) return -1;
+  if (d.tile && d.nnz > kTeamGridTileNnz && ctx->opt.precond == 0 && policy->kind == 0 && policy->fixed[0] == F64)
+    return -1;
+  return 0;
 }
 
 // Device tables of a launch of the team solver (systems as in build_plan).

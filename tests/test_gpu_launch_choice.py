@@ -50,3 +50,14 @@ def test_two_large_systems_as_teams(M):
         pol = ctx.policy_fixed((4, 4, 4, 4))
         took.append(_median(lambda: ctx.solve_batched(mats, bs, xs, [0.0] * 2, [30] * 2, pol)))
     assert took[0] < 2 * took[1]
+
+
+def test_a_system_beyond_the_whole_grid_team(M):
+    A = I.poisson2d(1800)  # 3.24e6 rows, just below 2^24 nonzeros
+    b = torch.as_tensor(np.random.default_rng(0).uniform(-1, 1, A[0])).cuda()
+    took = []
+    for stepped in (0, 2):
+        ctx = M.Context(0, M.Options(min_k=0, stepped=stepped))
+        mat, x, pol = ctx.matrix(_dev(A)), torch.zeros_like(b), ctx.policy_fixed((2, 4, 4, 4))
+        took.append(_median(lambda: ctx.solve(mat, b, x, 0.0, 30, pol)))
+    assert took[0] < 1.35 * took[1]
