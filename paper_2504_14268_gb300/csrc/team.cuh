@@ -63,6 +63,7 @@ struct TeamSmem {
   unsigned char* icring;          // ... and the ring of level blocks
   unsigned long long icbar[kIcBars];
   unsigned icuse;                 // ... blocks so far, modulo 2 kIcBars (the barriers' parity)
+  unsigned icissued;              // ... blocks of this application whose copies have been issued
   int icstop[2];                  // ... a wait gave up
   int icdone;                     // ... levels consumed in this application
   // the short scalar step (team_step_b): squared thresholds ([0]: the tolerance) as bit patterns
@@ -690,6 +691,7 @@ __device__ __noinline__ void ic_levels_team(const Launch& L, TeamSmem& t) {
           while (have < need && !wait_over(L, t, t0, ++spins)) have = lds_acquire(done);
           if (have >= need) {
             const unsigned bar = bars + 8u * ((use0 + (unsigned)(l0 + j)) % kIcBars);
+            t.icissued = (unsigned)(l0 + j + 1);
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(size * 16) : "memory");
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                              ring + 16u * (unsigned)to),
@@ -719,11 +721,12 @@ __device__ __noinline__ void ic_levels_team(const Launch& L, TeamSmem& t) {
       if (lane == 0) t.icstop[l & 1] = *(volatile int*)&t.bad;
       __syncwarp();
       asm volatile("bar.sync 1, %0;" ::"r"(nw * 32 + 32) : "memory");
-      if (*(volatile int*)&t.icstop[l & 1]) break;
+      if (*(volatile int*)&t.icstop[l & 1]) return;
       if (lane == 0) sts_release(smem_u32(&t.icdone), l);
     }
     if (lane == 0) {
       t.icuse = (use0 + (unsigned)nl) % (2u * kIcBars);
+      t.icissued = 0;
       sts_release(smem_u32(&t.icdone), 0);  // (the producer has issued the last block)
     }
     return;
@@ -753,6 +756,20 @@ __device__ __noinline__ void ic_levels_team(const Launch& L, TeamSmem& t) {
     }
     asm volatile("bar.sync 1, %0;" ::"r"(nw * 32 + 32) : "memory");
     blk = ring + 16u * (unsigned)h.z;
+  }
+}
+
+// After a wait that gave up: waits for the block copies still in flight, so that none lands in shared
+// memory that has passed to another CTA. A barrier of the ring was last used by one of the last kIcBars
+// blocks issued. (A copy needs nothing of the other CTAs; the limit is far beyond what it takes.)
+__device__ __noinline__ void ic_drain(TeamSmem& t) {
+  if (threadIdx.x != 0) return;
+  const unsigned n = t.icissued;
+  for (unsigned l = n > (unsigned)kIcBars ? n - kIcBars : 0u; l < n; ++l) {
+    const unsigned use = t.icuse + l;
+    const long long t0 = clock64();
+    while (!mbar_try_wait(&t.icbar[use % kIcBars], (use / kIcBars) & 1u))
+      if (clock64() - t0 > 100000000ll) return;
   }
 }
 
@@ -1244,6 +1261,7 @@ __global__ void __launch_bounds__(kTT, 1) cg_team(const __grid_constant__ Launch
     mbar_init(t.pbar + 1, (unsigned)size);
     for (int i = 0; i < kIcBars; ++i) mbar_init(&t.icbar[i], 1);
     t.icuse = 0;
+    t.icissued = 0;
     t.icdone = 0;
     mbar_fence_init();
   }
@@ -1338,10 +1356,16 @@ __global__ void __launch_bounds__(kTT, 1) cg_team(const __grid_constant__ Launch
     __syncthreads();
   }
   const bool ok = solve_team<CL, IC>(L, t, sid);
-  if (IC && !ok)  // a wait gave up: let the block copies in flight land first
-    for (int i = 0; i < 1000; ++i) __nanosleep(1000);
-  // no CTA of a cluster leaves while a peer may still write into its shared memory
-  if constexpr (CL) cluster_sync_all();
+  if constexpr (IC) {
+    if (!ok) ic_drain(t);
+  }
+  // no CTA of a cluster leaves while a peer may still write into its shared memory; after a wait that gave
+  // up, messages that nobody waits for any more (a microsecond each) get time to land
+  if constexpr (CL) {
+    cluster_sync_all();
+    if (!ok)
+      for (int i = 0; i < 100; ++i) __nanosleep(1000);
+  }
 }
 
 // Launches a cluster form of the kernel.
