@@ -1423,13 +1423,9 @@ mpcg_status mpcg_matrix_set_schedule(mpcg_matrix_t A, int32_t fmt, int32_t sched
   return MPCG_OK;
 }
 
-mpcg_status mpcg_spmv(mpcg_ctx_t ctx, mpcg_matrix_t A, int32_t fmt, const double* x, double* y, int32_t reps,
-                      double* ms_per_rep, void* stream) {
-  if (!ctx || !A || !x || !y) return fail(ctx, MPCG_ERR_INVALID_ARG, "NULL argument");
-  if (!valid_fmt(fmt)) return fail(ctx, MPCG_ERR_INVALID_ARG, "bad format %d", fmt);
-  if (!is_device_ptr(x) || !is_device_ptr(y)) return fail(ctx, MPCG_ERR_INVALID_ARG, "x and y must be device pointers");
-  cudaSetDevice(ctx->device);
-  cudaStream_t s = (cudaStream_t)stream;
+// y = A x in format fmt, `reps` products timed. tile_ok: an fp64 product may come from warp tiles.
+static mpcg_status run_spmv(mpcg_ctx_t ctx, mpcg_matrix_t A, int32_t fmt, const double* x, double* y, int32_t reps,
+                            double* ms_per_rep, bool tile_ok, cudaStream_t s) {
   const int n = A->dm.n;
   CK(ctx, ctx->spmv_x.ensure(4 * (size_t)n + 16));
   CK(ctx, ctx->spmv_q.ensure(8 * (size_t)n + 16));
@@ -1441,9 +1437,10 @@ mpcg_status mpcg_spmv(mpcg_ctx_t ctx, mpcg_matrix_t A, int32_t fmt, const double
   S.q = ctx->spmv_q.p;
   if (fmt != F64) CK(ctx, launch_to_format(x, S.plow, n, fmt, s));
   // The launch shape the solver uses for this matrix: with the stream ring when any format
-  // of the matrix uses the stream schedule.
+  // of the matrix uses the stream schedule; or the fp64 product from warp tiles, which of the solves only
+  // the stepped one with a fixed policy and fp64 products runs.
   const bool stream_shape = A->force_stream_shape || uses_stream(A->dm);
-  const bool tile = fmt == F64 && A->dm.tile && A->dm.sched[F64] == SCHED_VLOAD;
+  const bool tile = tile_ok && fmt == F64 && A->dm.tile && A->dm.sched[F64] == SCHED_VLOAD;
   const int grid = ctx->nsm * (tile ? ctx->socc_t : stream_shape ? ctx->occ_s : ctx->occ);
   const int stage = stream_shape ? kStageBytes : 0;
   CK(ctx, ctx->spmv_err.ensure(sizeof(unsigned)));
@@ -1467,6 +1464,15 @@ mpcg_status mpcg_spmv(mpcg_ctx_t ctx, mpcg_matrix_t A, int32_t fmt, const double
   if (herr) return fail(ctx, MPCG_ERR_TIMEOUT, "a bulk-copy wait of the product exceeded its limit");
   if (ms_per_rep) *ms_per_rep = ms / reps;
   return MPCG_OK;
+}
+
+mpcg_status mpcg_spmv(mpcg_ctx_t ctx, mpcg_matrix_t A, int32_t fmt, const double* x, double* y, int32_t reps,
+                      double* ms_per_rep, void* stream) {
+  if (!ctx || !A || !x || !y) return fail(ctx, MPCG_ERR_INVALID_ARG, "NULL argument");
+  if (!valid_fmt(fmt)) return fail(ctx, MPCG_ERR_INVALID_ARG, "bad format %d", fmt);
+  if (!is_device_ptr(x) || !is_device_ptr(y)) return fail(ctx, MPCG_ERR_INVALID_ARG, "x and y must be device pointers");
+  cudaSetDevice(ctx->device);
+  return run_spmv(ctx, A, fmt, x, y, reps, ms_per_rep, true, (cudaStream_t)stream);
 }
 
 namespace {
@@ -1530,7 +1536,8 @@ mpcg_status autotune_timed(mpcg_ctx_t ctx, mpcg_matrix_t A, int32_t reps, void* 
   auto time_it = [&](int f, int sched, int lanes, double& ms) -> mpcg_status {
     mpcg_status st = mpcg_matrix_set_schedule(A, f, sched, lanes);
     if (st != MPCG_OK) return st;
-    return mpcg_spmv(ctx, A, f, x.as<double>(), y.as<double>(), reps, &ms, stream);
+    // the direct loads also where warp tiles are faster: tables, schedules and batches run those
+    return run_spmv(ctx, A, f, x.as<double>(), y.as<double>(), reps, &ms, false, (cudaStream_t)stream);
   };
   // Configuration P: every format on the sub-warp vector schedule, no stream ring.
   int bestP[NFMT];
