@@ -588,6 +588,19 @@ TeamEstimate team_sizes(mpcg_ctx_t ctx, const std::vector<SysIn>& in, int most, 
   return e;
 }
 
+// Entries of the Q-table and of its visit counts that a team holds in shared memory (none when the table
+// is larger than kTeamQBytes), and their room in fp64 words.
+struct TeamTable {
+  int q, v;
+  size_t words;
+};
+TeamTable team_table(mpcg_ctx_t ctx, mpcg_policy_t policy) {
+  const int S = ctx->opt.b_bins * ctx->opt.r_bins, joint = ctx->opt.joint ? 1 : 0;
+  const bool held = policy->kind == 2 && 8 * qtable_size(S, ctx->opt.nprec, joint) <= kTeamQBytes;
+  const int q = held ? (int)qtable_size(S, ctx->opt.nprec, joint) : 0, v = held ? (int)visits_size(S, joint) : 0;
+  return TeamTable{q, v, (size_t)(q + (v + 1) / 2 + 1)};
+}
+
 // The team solver takes a launch when every product of its matrices runs one of the two
 // row-length schedules and the options are those it implements. Returns the CTAs per cluster, 0
 // for the whole grid on one system, -1 when another kernel takes the launch. Training rounds and the
@@ -599,8 +612,7 @@ int team_rule(mpcg_ctx_t ctx, const std::vector<SysIn>& in, mpcg_policy_t policy
   const int nsys = (int)in.size();
   if (nsys < 1 || train || ctx->max_cluster < 1 || ctx->opt.variant != 0 || ctx->opt.batch_mode == 2) return -1;
   const bool ic = ctx->opt.precond == 2;
-  const int S = ctx->opt.b_bins * ctx->opt.r_bins, joint = ctx->opt.joint ? 1 : 0;
-  const size_t table = policy->kind == 2 ? (size_t)kTeamQBytes + 4 * (size_t)visits_size(S, joint) : 0;
+  const size_t table = 8 * team_table(ctx, policy).words;
   for (const SysIn& s : in) {  // the ring, the vector and the table fit a CTA's shared memory
     const size_t need = team_ic_bytes(s.A) + table + 256;
     if (ic && (!s.A->icwarps || need > team_max_heap())) return -1;
@@ -692,10 +704,7 @@ mpcg_status build_team_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& 
   // vectors of the largest share of rows (even shares of nnz + 4 n; of rows half as long as the
   // mean, as at grid boundaries, a share holds that many). A CTA whose rows exceed what was given
   // keeps its vectors in global memory.
-  const int S = ctx->opt.b_bins * ctx->opt.r_bins, joint = ctx->opt.joint ? 1 : 0;
-  const bool table = policy->kind == 2 && 8 * qtable_size(S, ctx->opt.nprec, joint) <= kTeamQBytes;
-  const int team_q = table ? (int)qtable_size(S, ctx->opt.nprec, joint) : 0;
-  const int team_v = table ? (int)visits_size(S, joint) : 0;
+  const TeamTable table = team_table(ctx, policy);
   size_t heap = 0;
   bool tiles = false;
   for (int i = 0; i < nsys; ++i) {
@@ -711,7 +720,7 @@ mpcg_status build_team_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& 
     // product tiles (24 iterations of 64^3 27-point CG: fp64 1.36 -> 1.08 ms, fp32 1.08 -> 0.80;
     // 36^3, whose columns fit: tiles 0.51 ms, direct loads 0.47).
     const size_t tile = (size_t)kTeamTileWarp * (kTeamThreads / 32) + 32;
-    const size_t other = (cluster ? 0 : 32 * (size_t)ctx->nsm) + 8 * (size_t)(team_q + (team_v + 1) / 2 + 1) + 256;
+    const size_t other = (cluster ? 0 : 32 * (size_t)ctx->nsm) + 8 * table.words + 256;
     if (need + idx <= kTeamIndexHeap) {
       need += idx;
     } else if (A->dm.tile && need + tile + other <= team_max_heap()) {
@@ -720,7 +729,7 @@ mpcg_status build_team_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& 
     }
     heap = std::max(heap, need);
   }
-  heap += (cluster ? 0 : 8 * 4 * (size_t)grid) + 8 * (size_t)(team_q + (team_v + 1) / 2 + 1);
+  heap += (cluster ? 0 : 8 * 4 * (size_t)grid) + 8 * table.words;
   heap = std::min((heap + 127) / 128 * 128, team_max_heap());
   CK(ctx, pl.st.ensure(sizeof(SysState) * nsys));
   const size_t sys_bytes = (sizeof(DevSys) * nsys + 15) / 16 * 16, cta_bytes = sizeof(int4) * ctas.size();
@@ -745,8 +754,8 @@ mpcg_status build_team_plan(mpcg_ctx_t ctx, Plan& pl, const std::vector<SysIn>& 
   L.res = reinterpret_cast<mpcg_result*>(out + pl.xch_bytes + 16);
   L.team_heap = (int)heap;
   L.tile = tiles ? 1 : 0;
-  L.team_q = team_q;
-  L.team_v = team_v;
+  L.team_q = table.q;
+  L.team_v = table.v;
   const mpcg_status st = fill_policy(ctx, policy, L.pol);
   if (st != MPCG_OK) return st;
   L.opt = ctx->ov;
