@@ -11,6 +11,7 @@
 #include <memory>
 #include <numeric>
 #include <map>
+#include <new>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -448,15 +449,20 @@ mpcg_status ensure_ic0(mpcg_ctx_t ctx, mpcg_matrix_s* M, cudaStream_t s) {
   // place in the ring, bytes of a group}, then per group each lane's {row, diagonal} (row 0xffff:
   // padding), columns and values, quad q of lane t at 32 q + t; padding entries are 0 in column n.
   // Only for systems whose vector fits a CTA's shared memory beside a ring of blocks and whose
-  // levels are even enough not to be blown up by the padding.
+  // levels are even enough not to be blown up by the padding. Where there is no memory for it (up to 64
+  // bytes a nonzero, here and on the device) the other kernels do without.
   std::vector<float> hF;
   std::vector<unsigned char> blob;
   std::vector<IcBlock> desc;
   size_t block_max = 0, groups_max = 0;
   bool packed = n > 0 && n <= kTeamIcRows;
   if (packed) {
-    hF.resize((size_t)std::max(nnz, 1LL));
-    CK(ctx, cudaMemcpy(hF.data(), M->icf.p, 4 * (size_t)nnz, cudaMemcpyDeviceToHost));
+    try {
+      hF.resize((size_t)std::max(nnz, 1LL));
+    } catch (const std::bad_alloc&) {
+      packed = false;
+    }
+    if (packed) CK(ctx, cudaMemcpy(hF.data(), M->icf.p, 4 * (size_t)nnz, cudaMemcpyDeviceToHost));
   }
   auto pack_levels = [&](int depth, bool lower) {  // lev, perm: this direction's levels and order
     std::vector<int> start(depth + 1, 0);
@@ -515,7 +521,11 @@ mpcg_status ensure_ic0(mpcg_ctx_t ctx, mpcg_matrix_s* M, cudaStream_t s) {
   }
   mpcg_status ls = sort_by_level(depth, M->icpf, M->icof, M->icwf, M->nlevf);
   if (ls != MPCG_OK) return ls;
-  if (packed) pack_levels(depth, true);
+  try {
+    if (packed) pack_levels(depth, true);
+  } catch (const std::bad_alloc&) {
+    packed = false;
+  }
   depth = 0;
   for (int i = n - 1; i >= 0; --i) {  // L^T w = y: row i reads w_j, j > i, over its upper entries
     int l = 0;
@@ -525,7 +535,11 @@ mpcg_status ensure_ic0(mpcg_ctx_t ctx, mpcg_matrix_s* M, cudaStream_t s) {
   }
   ls = sort_by_level(depth, M->icpb, M->icob, M->icwb, M->nlevb);
   if (ls != MPCG_OK) return ls;
-  if (packed) pack_levels(depth, false);
+  try {
+    if (packed) pack_levels(depth, false);
+  } catch (const std::bad_alloc&) {
+    packed = false;
+  }
   // The ring beside the vector; from some 21,500 rows it is smaller than kTeamIcRing, and systems with
   // wide levels (27-point grids from 30^3, 7-point from 31^3) no longer fit it: other kernels take those.
   const size_t fit = kTeamIcShared / 16 * 16 - 8 * (((size_t)n + 2) / 2);
@@ -534,13 +548,16 @@ mpcg_status ensure_ic0(mpcg_ctx_t ctx, mpcg_matrix_s* M, cudaStream_t s) {
     for (size_t l = 0; l + 1 < desc.size(); ++l)  // each block names the next one's place
       memcpy(blob.data() + (size_t)desc[l].from * 16 + 8, &desc[l + 1].at, 4);
     static_assert(sizeof(IcBlock) == sizeof(int4), "the kernel reads blocks as int4");
-    M->icring = cap * 16;
-    CK(ctx, M->icblob.ensure(blob.size()));
-    CK(ctx, M->icdesc.ensure(sizeof(IcBlock) * desc.size()));
-    CK(ctx, cudaMemcpy(M->icblob.p, blob.data(), blob.size(), cudaMemcpyHostToDevice));
-    CK(ctx, cudaMemcpy(M->icdesc.p, desc.data(), sizeof(IcBlock) * desc.size(), cudaMemcpyHostToDevice));
-    M->icwarps = (int)std::min<size_t>(groups_max, kTeamThreads / 32 - 2);  // (one warp waits, one copies)
-    M->bytes += (long long)blob.size();
+    if (M->icblob.ensure(blob.size()) != cudaSuccess ||
+        M->icdesc.ensure(sizeof(IcBlock) * desc.size()) != cudaSuccess) {
+      cudaGetLastError();
+    } else {
+      CK(ctx, cudaMemcpy(M->icblob.p, blob.data(), blob.size(), cudaMemcpyHostToDevice));
+      CK(ctx, cudaMemcpy(M->icdesc.p, desc.data(), sizeof(IcBlock) * desc.size(), cudaMemcpyHostToDevice));
+      M->icring = cap * 16;
+      M->icwarps = (int)std::min<size_t>(groups_max, kTeamThreads / 32 - 2);  // (one warp waits, one copies)
+      M->bytes += (long long)(blob.size() + sizeof(IcBlock) * desc.size());
+    }
   }
   M->ic_ready = true;
   M->bytes += 4 * nnz + 12LL * n;
