@@ -146,7 +146,8 @@ typedef struct {
                             * rho can move the state to the next bin (5e-3)              */
   int32_t stepped;         /* single solves (mpcg_solve): 0 = automatic (stepped for systems
                             * of at least 2^24 nonzeros without IC(0)), 1 = one launch of
-                            * a team (a cluster or the whole grid), 2 = stepped: one kernel per phase of the
+                            * a team (a cluster, the whole grid or the persistent kernel,
+                            * by size), 2 = stepped: one kernel per phase of the
                             * iteration, repeated on the device by a conditional while-loop
                             * CUDA graph, 3 = the same kernels with each pass launched by the
                             * host, which reads the phase back after every pass (for tools
@@ -264,7 +265,9 @@ mpcg_status mpcg_matrix_autotune(mpcg_ctx_t ctx, mpcg_matrix_t A, int32_t reps, 
  * l_ji at (i, j) for j > i. Needs strictly increasing column indices in every row, a
  * diagonal entry in every row and a symmetric pattern (INVALID_ARG otherwise); a
  * non-positive pivot (IC(0) exists for M-matrices, not for every SPD matrix) is INVALID_ARG
- * "breaks down". Synchronises `stream`. */
+ * "breaks down". Kept with the matrix: 4 bytes per nonzero and 12 per row, and for up to 32768
+ * rows a copy laid out by levels (up to 64 bytes per nonzero; a matrix for which there is no
+ * memory goes without). Synchronises `stream`. */
 mpcg_status mpcg_matrix_ic0(mpcg_ctx_t ctx, mpcg_matrix_t A, float* factor, void* stream);
 /* Dependency levels of the two triangular substitutions of a CSR pattern (host pointers,
  * no device work; the scheduling analysis of the IC(0) substitutions): level_lower[i] =
@@ -286,13 +289,16 @@ mpcg_status mpcg_csr_levels(int32_t n, const int32_t* row_ptr, const int32_t* co
  * of the window of x that the CTA's rows read, when it fits (otherwise from x), `lanes` = 1,
  * for matrices whose column indices increase in every row). In schedules 0, 2 and 4 a row
  * longer than 1024 nonzeros (a power-law hub) is summed by a whole CTA after the CTA's other
- * rows.
+ * rows (one-launch team solves: fp64 and correctly rounded rows over 32 by a warp, over 512 by
+ * the CTA).
  * INVALID_ARG for other combinations and for a stream tile that does not fit its
  * shared-memory stage. */
 mpcg_status mpcg_matrix_set_schedule(mpcg_matrix_t A, int32_t fmt, int32_t sched, int32_t lanes);
 
 /* y = fl_fmt(A fl_fmt(x)) with the matrix's schedule for `fmt` (op 1 of Section 4.2 on its
- * own; x and y fp64 device vectors of length n). `reps` > 1 repeats the product (for timing);
+ * own; x and y fp64 device vectors of length n; the fp64 product of schedule 2 from warp tiles
+ * where no 32 rows exceed 896 nonzeros, as in stepped solves of a fixed policy with fp64
+ * products). `reps` > 1 repeats the product (for timing);
  * if ms_per_rep is non-NULL it receives the mean device time of one product. */
 mpcg_status mpcg_spmv(mpcg_ctx_t ctx, mpcg_matrix_t A, int32_t fmt, const double* x, double* y,
                       int32_t reps, double* ms_per_rep, void* stream);
@@ -391,7 +397,10 @@ mpcg_status mpcg_solve_noalloc(mpcg_ctx_t ctx, mpcg_matrix_t A, const double* b,
  * from x_0 = 0 on a private copy of the tables, updating the copy online; at the end of the
  * round the shared tables are rebuilt by replaying every recorded transition (system 0..
  * nsys-1, then iteration order) onto the round-start tables. With nsys = 1 this is
- * Algorithm 1. `inout` is a QTABLE policy updated in place. iters_out (optional, host,
+ * Algorithm 1. The same seed, options and systems give the same table bit for bit; the sums'
+ * order, and with it last bits that a learner can magnify, depends on the systems of the call
+ * (rounds of several run in lockstep, one alone in the persistent kernel, whatever
+ * options.batch_mode = 0 or a solve would choose). `inout` is a QTABLE policy updated in place. iters_out (optional, host,
  * [episodes][nsys]) receives each episode's iteration count. b[i]: device pointers. */
 mpcg_status mpcg_train_qtable(mpcg_ctx_t ctx, int32_t nsys, const mpcg_matrix_t* A,
                               const double* const* b, double tol, int32_t t_max, int32_t episodes,

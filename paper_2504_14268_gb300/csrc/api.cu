@@ -59,7 +59,11 @@ bool is_device_ptr(const void* p) {
 constexpr long long kTimeoutCycles = 4000000000ll;  // about two seconds at 2 GHz per wait
 constexpr double kTileMinMean = 14.0;              // mean row length from which warp tiles pay
 constexpr int kTeamBatchCluster = 8;               // cluster of a batch's teams
-constexpr long long kTeamCtaWork = 8192;           // a team has a CTA per so much work (nnz + 4 n)
+// A team has a CTA per so much work (nnz + 4 n). Half as many CTAs are slower from some 1,000 rows on; more
+// would be faster from there to some 6,000 rows, and slower below (60 iterations of fp64 CG with 2048 /
+// 8192 / 16384: five-point 16^2 0.44 / 0.39 / 0.39 ms, 32^2 0.47 / 0.56 / 0.63, 64^2 0.51 / 0.65 / 0.76,
+// 90^2, a full cluster, 0.65 / 0.65 / 0.72; 7-point 18^3 0.56 / 0.67 / 0.88; 27-point 12^3 0.63 / 0.64 / 0.72).
+constexpr long long kTeamCtaWork = 8192;
 constexpr long long kTeamGridWork = 160 * 1000;    // from here a single system takes the whole grid ...
 constexpr int kTeamGridRows = 1200 * 1000;         // ... up to so many rows,
 constexpr int kTeamGridRowsPlain = 1400 * 1000;    // ... with fp64 or fp32 products only up to so many,
@@ -642,7 +646,9 @@ int team_rule(mpcg_ctx_t ctx, const std::vector<SysIn>& in, mpcg_policy_t policy
     // by the estimate below sooner than the lockstep kernel: per CTA 0.84 ns a unit of cost and 10 us
     // an iteration, against 100 us an iteration and the matrices at 4 TB/s (48 systems of 1,000 to
     // 60,000 rows, 60 iterations: 5.6 against 7.6 ms; 512 systems of 6e8 nonzeros, 5,000
-    // iterations: 71 against 10.7 s). IC(0) substitutions run in the team whenever they can. Against the
+    // iterations: 71 against 10.7 s; of 45 batches of 2 to 128 systems none ended more than 6% later than
+    // in lockstep, most a multiple sooner). IC(0) substitutions run in the team whenever they can (4 to 300
+    // systems of 900 to 19,600 rows: 2.3 to 8.3 times as fast as lockstep). Against the
     // persistent teams (batch_mode 1), which share the whole grid among a few systems: 85 us an iteration
     // and the matrices at 5 TB/s, the team's figure without its margin (30 iterations of 27-point fp64 CG:
     // two 64^3 systems 17.0 ms in clusters of 16, 3.5 ms in persistent teams; eight of 30^3 2.3 against

@@ -23,8 +23,8 @@ constexpr int kTileEntries = 896;   // nonzeros of a warp's tile (32 rows) of th
 constexpr int kTileWarpBytes = 4 * (kTileEntries + 8) + 8 * (kTileEntries + 2);  // columns, fp64 values
 constexpr int kTileBytes = kTileWarpBytes * (kThreads / 32);
 // Threads per CTA of the team solver: 512 leave 128 registers for loads in flight, and a barrier takes 30
-// to 79 cycles with the warps it holds (against 1024: training on 8 systems 2.48 -> 2.41 ms, IC(0) on a
-// 28^3 27-point system 4.77 -> 4.36, a 160,000-row graph 0.94 -> 0.91).
+// to 79 cycles with the warps it holds (against 1024: IC(0) on a 28^3 27-point system 4.77 -> 4.36 ms, a
+// 160,000-row graph 0.94 -> 0.91).
 constexpr int kTeamThreads = 512;
 constexpr int kTeamTileWarp = 7232; // bytes of a warp's product tile
 constexpr int kTeamIcBars = 32;    // level blocks of the IC(0) substitutions in flight at most

@@ -499,7 +499,8 @@ __device__ void spmv_vload(const DevSys& S, const VT* __restrict__ vals, const V
 // One thread per row from warp tiles, fp64: a warp takes 32 consecutive rows, copies their contiguous
 // columns and values to its own part of shared memory with coalesced asynchronous 16-byte copies
 // (no registers in between), and every lane then walks its row there, in column order as
-// spmv_vload does, so the sums are the same bit for bit. What bounds the direct loads of rows of
+// spmv_vload does, so the row sums are the same bit for bit (the stepped solve's nu is not: its CTAs' parts
+// are cut for two CTAs an SM instead of four). What bounds the direct loads of rows of
 // 16 and more nonzeros is the L1: a warp's 16-byte loads fall on 32 different lines, some 700 line
 // look-ups per 32 rows of 27 nonzeros against 150 this way. Two thirds of the gathers miss the L1,
 // so a row takes as many round trips to L2 as it has batches of gathers: the kernels that run this

@@ -1057,8 +1057,8 @@ __device__ __noinline__ TeamOk team_restart64(const Launch& L, TeamSmem& t, Team
   team_publish<CL>(L, t, T);
   const double rr = team_true_res(t);
   const TeamDot u = team_use_r<CL, IC>(L, t, T, -1, -1, true);
-    T = u.T;
-    const DotAcc sg = u.sg;
+  T = u.T;
+  const DotAcc sg = u.sg;
   const double v[2] = {warp_sum(rr), warp_dot(sg, false)};
   team_exchange<CL, 2>(L, t, T, v);
   if (threadIdx.x == 0) t.stale = 0;

@@ -204,7 +204,7 @@ class Options:
     batch_mode: int = 0
     precond: int = 0  # 0: M = I; 1: Jacobi; 2: fp32 IC(0) (factor kept with the matrix)
     edge_tol: float = 5e-3  # greedy decisions this close (relative) to a residual-bin edge are counted
-    stepped: int = 0  # single solves: 0 automatic, 1 persistent launch, 2 one kernel per phase in a graph loop
+    stepped: int = 0  # single solves: 0 automatic, 1 one launch (team or persistent), 2 one kernel per phase in a graph loop
     variant: int = 0  # 0: the CG of Section 3; 1: the single-reduction iteration (lockstep / stepped kernels)
     joint: int = 0  # tabular policies: 1 = one table over the joint actions, Q[S][nprec^4], visits[S]
 
