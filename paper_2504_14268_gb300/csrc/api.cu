@@ -414,6 +414,9 @@ mpcg_status ensure_ic0(mpcg_ctx_t ctx, mpcg_matrix_s* M, cudaStream_t s) {
   const long long nnz = M->dm.nnz;
   CK(ctx, M->icf.ensure(4 * (size_t)std::max(nnz, 1LL)));
   CK(ctx, M->icd.ensure(4 * (size_t)std::max(n, 1)));
+  std::vector<int> hrp(n + 1), hci((size_t)std::max(nnz, 1LL));
+  CK(ctx, cudaMemcpy(hrp.data(), M->dm.rp, 4 * (size_t)(n + 1), cudaMemcpyDeviceToHost));
+  if (nnz) CK(ctx, cudaMemcpy(hci.data(), M->dm.ci, 4 * (size_t)nnz, cudaMemcpyDeviceToHost));
   DevBuf done, err;
   CK(ctx, done.ensure(4 * (size_t)std::max(n, 1)));
   CK(ctx, err.ensure(sizeof(unsigned)));
@@ -421,101 +424,35 @@ mpcg_status ensure_ic0(mpcg_ctx_t ctx, mpcg_matrix_s* M, cudaStream_t s) {
   CK(ctx, cudaMemsetAsync(err.p, 0, sizeof(unsigned), s));
   CK(ctx, launch_ic0_factor(n, M->dm.rp, M->dm.ci, M->dm.v64, M->icf.as<float>(), M->icd.as<int>(),
                             done.as<unsigned>(), err.as<unsigned>(), kTimeoutCycles, ctx->nsm, s));
-  unsigned bits = 0;
-  CK(ctx, cudaMemcpyAsync(&bits, err.p, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-  CK(ctx, cudaStreamSynchronize(s));
-  if (bits) {
-    M->ic_fail = bits;
-    return ic0_error(ctx, bits);
-  }
-  // level schedule of the substitutions (host pass over the pattern): rows sorted by level,
-  // stable in the row index
-  std::vector<int> hrp(n + 1), hci((size_t)std::max(nnz, 1LL)), hdp(std::max(n, 1));
-  CK(ctx, cudaMemcpy(hrp.data(), M->dm.rp, 4 * (size_t)(n + 1), cudaMemcpyDeviceToHost));
-  if (nnz) CK(ctx, cudaMemcpy(hci.data(), M->dm.ci, 4 * (size_t)nnz, cudaMemcpyDeviceToHost));
-  if (n) CK(ctx, cudaMemcpy(hdp.data(), M->icd.p, 4 * (size_t)n, cudaMemcpyDeviceToHost));
-  std::vector<int> lev(std::max(n, 1)), perm(std::max(n, 1));
-  auto sort_by_level = [&](int depth, DevBuf& out, DevBuf& starts, int& width, int& nlev) -> mpcg_status {
-    std::vector<int> cnt(depth + 1, 0);
-    for (int i = 0; i < n; ++i) ++cnt[lev[i] + 1];
-    width = 0;
-    for (int l = 0; l < depth; ++l) width = std::max(width, cnt[l + 1]);
-    for (int l = 0; l < depth; ++l) cnt[l + 1] += cnt[l];
-    CK(ctx, starts.ensure(4 * (size_t)(depth + 1)));
-    CK(ctx, cudaMemcpy(starts.p, cnt.data(), 4 * (size_t)(depth + 1), cudaMemcpyHostToDevice));
-    nlev = depth;
-    for (int i = 0; i < n; ++i) perm[cnt[lev[i]]++] = i;
-    CK(ctx, out.ensure(4 * (size_t)std::max(n, 1)));
-    if (n) CK(ctx, cudaMemcpy(out.p, perm.data(), 4 * (size_t)n, cudaMemcpyHostToDevice));
-    return MPCG_OK;
-  };
-  // The team solver's form: per level a block {groups of 32 rows, quads of entries, the next block's
-  // place in the ring, bytes of a group}, then per group each lane's {row, diagonal} (row 0xffff:
-  // padding), columns and values, quad q of lane t at 32 q + t; padding entries are 0 in column n.
-  // Only for systems whose vector fits a CTA's shared memory beside a ring of blocks and whose
-  // levels are even enough not to be blown up by the padding. Where there is no memory for it (up to 64
-  // bytes a nonzero, here and on the device) the other kernels do without.
-  std::vector<float> hF;
-  std::vector<unsigned char> blob;
-  std::vector<IcBlock> desc;
-  size_t block_max = 0, groups_max = 0;
-  bool packed = n > 0 && n <= kTeamIcRows;
-  if (packed) {
-    try {
-      hF.resize((size_t)std::max(nnz, 1LL));
-    } catch (const std::bad_alloc&) {
-      packed = false;
-    }
-    if (packed) CK(ctx, cudaMemcpy(hF.data(), M->icf.p, 4 * (size_t)nnz, cudaMemcpyDeviceToHost));
-  }
-  auto pack_levels = [&](int depth, bool lower) {  // lev, perm: this direction's levels and order
-    std::vector<int> start(depth + 1, 0);
-    for (int i = 0; i < n; ++i) ++start[lev[i] + 1];
-    for (int l = 0; l < depth; ++l) start[l + 1] += start[l];
-    for (int l = 0; l < depth && packed; ++l) {
-      const int cnt = start[l + 1] - start[l], ng = (cnt + 31) / 32;
-      auto first = [&](int i) { return lower ? hrp[i] : hdp[i] + 1; };
-      auto last = [&](int i) { return lower ? hdp[i] : hrp[i + 1]; };
-      int len = 0;
-      for (int x = start[l]; x < start[l + 1]; ++x) len = std::max(len, last(perm[x]) - first(perm[x]));
-      // quads of entries: one, two, or a multiple of four
-      const int quads = len <= 4 ? 1 : len <= 8 ? 2 : (len + 15) / 16 * 4;
-      const size_t group = 256 + 768 * (size_t)quads, bytes = 16 + ng * group;
-      block_max = std::max(block_max, bytes);
-      groups_max = std::max(groups_max, (size_t)ng);
-      if (3 * block_max > kTeamIcRing || blob.size() + bytes > 64ull * nnz + (1u << 20)) {
-        packed = false;
-        return;
+  // While the device factors: the level schedule of the substitutions (host pass over the pattern), rows
+  // sorted by level, stable in the row index. (A row without a diagonal entry, which the factorization
+  // refuses, has none of its entries above it here.)
+  std::vector<int> hdp(std::max(n, 1));
+  for (int i = 0; i < n; ++i) {
+    hdp[i] = hrp[i + 1] - 1;
+    for (int e = hrp[i]; e < hrp[i + 1]; ++e)
+      if (hci[e] == i) {
+        hdp[i] = e;
+        break;
       }
-      const size_t at = blob.size();
-      desc.push_back(IcBlock{(int)(at / 16), (int)(bytes / 16), 0, 0});
-      blob.resize(at + bytes, 0);
-      unsigned char* o = blob.data() + at;
-      ((int*)o)[0] = ng;
-      ((int*)o)[1] = quads;
-      ((int*)o)[3] = (int)group;
-      for (int x = 0; x < ng * 32; ++x) {
-        const int t = x % 32;
-        unsigned char* og = o + 16 + (size_t)(x / 32) * group;
-        uint2* meta = (uint2*)og;
-        unsigned short* cols = (unsigned short*)(og + 256);
-        float* vals = (float*)(og + 256 + 256 * (size_t)quads);
-        for (int k = 0; k < 4 * quads; ++k) cols[(k / 4 * 32 + t) * 4 + k % 4] = (unsigned short)n;
-        if (x >= cnt) {
-          meta[t] = make_uint2(0xffffu, 0u);
-          continue;
-        }
-        const int i = perm[start[l] + x], e0 = first(i), e1 = last(i);
-        unsigned bits;
-        memcpy(&bits, &hF[hdp[i]], 4);
-        meta[t] = make_uint2((unsigned)i, bits);
-        for (int k = 0; k < e1 - e0; ++k) {
-          cols[(k / 4 * 32 + t) * 4 + k % 4] = (unsigned short)hci[e0 + k];
-          vals[(k / 4 * 32 + t) * 4 + k % 4] = hF[e0 + k];
-        }
-      }
-    }
+  }
+  struct Levels {
+    std::vector<int> perm, start;  // rows in level order; each level's first position in it
+    int depth = 0, width = 0;
   };
+  auto sort_by_level = [&](const std::vector<int>& lev, int depth) {
+    Levels L;
+    L.depth = depth;
+    L.start.assign(depth + 1, 0);
+    for (int i = 0; i < n; ++i) ++L.start[lev[i] + 1];
+    for (int l = 0; l < depth; ++l) L.width = std::max(L.width, L.start[l + 1]);
+    for (int l = 0; l < depth; ++l) L.start[l + 1] += L.start[l];
+    std::vector<int> at(L.start);
+    L.perm.resize(std::max(n, 1));
+    for (int i = 0; i < n; ++i) L.perm[at[lev[i]]++] = i;
+    return L;
+  };
+  std::vector<int> lev(std::max(n, 1));
   int depth = 0;
   for (int i = 0; i < n; ++i) {  // L y = r: row i reads y_j, j < i, over its lower entries
     int l = 0;
@@ -523,13 +460,7 @@ mpcg_status ensure_ic0(mpcg_ctx_t ctx, mpcg_matrix_s* M, cudaStream_t s) {
     lev[i] = l;
     depth = std::max(depth, l + 1);
   }
-  mpcg_status ls = sort_by_level(depth, M->icpf, M->icof, M->icwf, M->nlevf);
-  if (ls != MPCG_OK) return ls;
-  try {
-    if (packed) pack_levels(depth, true);
-  } catch (const std::bad_alloc&) {
-    packed = false;
-  }
+  const Levels fwd = sort_by_level(lev, depth);
   depth = 0;
   for (int i = n - 1; i >= 0; --i) {  // L^T w = y: row i reads w_j, j > i, over its upper entries
     int l = 0;
@@ -537,10 +468,62 @@ mpcg_status ensure_ic0(mpcg_ctx_t ctx, mpcg_matrix_s* M, cudaStream_t s) {
     lev[i] = l;
     depth = std::max(depth, l + 1);
   }
-  ls = sort_by_level(depth, M->icpb, M->icob, M->icwb, M->nlevb);
-  if (ls != MPCG_OK) return ls;
+  const Levels bwd = sort_by_level(lev, depth);
+  // The team solver's form: per level a block {groups of 32 rows, quads of entries, the next block's
+  // place in the ring, bytes of a group}, then per group each lane's {row, diagonal} (row 0xffff:
+  // padding), columns and values, quad q of lane t at 32 q + t; padding entries are 0 in column n.
+  // Only for systems whose vector fits a CTA's shared memory beside a ring of blocks and whose
+  // levels are even enough not to be blown up by the padding. Where there is no memory for it (up to 64
+  // bytes a nonzero, here and on the device) the other kernels do without. All but the factor's values
+  // is laid out beside the factorization, too (after it: 80^2 five-point 1.10 ms, 28^3 27-point 12.2; beside
+  // it 0.90 and 11.1; with no blocks and the levels after it 0.83 and 9.9).
+  std::vector<float> hF;
+  std::vector<unsigned char> blob;
+  std::vector<IcBlock> desc;
+  std::vector<int> quads_of;  // of each block
+  size_t block_max = 0, groups_max = 0;
+  auto first = [&](int i, bool lower) { return lower ? hrp[i] : hdp[i] + 1; };
+  auto last = [&](int i, bool lower) { return lower ? hdp[i] : hrp[i + 1]; };
+  auto block_sizes = [&]() {
+    size_t total = 0;
+    for (const Levels* L : {&fwd, &bwd})
+      for (int l = 0; l < L->depth; ++l) {
+        const size_t ng = (L->start[l + 1] - L->start[l] + 31) / 32;
+        int len = 0;
+        for (int x = L->start[l]; x < L->start[l + 1]; ++x)
+          len = std::max(len, last(L->perm[x], L == &fwd) - first(L->perm[x], L == &fwd));
+        // quads of entries: one, two, or a multiple of four
+        quads_of.push_back(len <= 4 ? 1 : len <= 8 ? 2 : (len + 15) / 16 * 4);
+        const size_t bytes = 16 + ng * (256 + 768 * (size_t)quads_of.back());
+        block_max = std::max(block_max, bytes);
+        groups_max = std::max(groups_max, ng);
+        if (3 * block_max > kTeamIcRing || total + bytes > 64ull * nnz + (1u << 20)) return false;
+        desc.push_back(IcBlock{(int)(total / 16), (int)(bytes / 16), 0, 0});
+        total += bytes;
+      }
+    blob.resize(total, 0);
+    hF.resize((size_t)std::max(nnz, 1LL));
+    return true;
+  };
+  // f(row, its first and last entry, {row, diagonal}, columns and values of the lane's first quad), the
+  // next quads 128 entries on
+  auto each_row = [&](auto&& f) {
+    size_t b = 0;
+    for (const Levels* L : {&fwd, &bwd})
+      for (int l = 0; l < L->depth; ++l, ++b) {
+        unsigned char* o = blob.data() + (size_t)desc[b].from * 16;
+        const size_t quads = quads_of[b], group = 256 + 768 * quads;
+        for (int x = L->start[l]; x < L->start[l + 1]; ++x) {
+          const int t = (x - L->start[l]) % 32, i = L->perm[x];
+          unsigned char* og = o + 16 + (size_t)((x - L->start[l]) / 32) * group;
+          f(i, first(i, L == &fwd), last(i, L == &fwd), (uint2*)og + t, (unsigned short*)(og + 256) + 4 * t,
+            (float*)(og + 256 + 256 * quads) + 4 * t);
+        }
+      }
+  };
+  bool packed = n > 0 && n <= kTeamIcRows;
   try {
-    if (packed) pack_levels(depth, false);
+    packed = packed && block_sizes();
   } catch (const std::bad_alloc&) {
     packed = false;
   }
@@ -548,9 +531,55 @@ mpcg_status ensure_ic0(mpcg_ctx_t ctx, mpcg_matrix_s* M, cudaStream_t s) {
   // wide levels (27-point grids from 30^3, 7-point from 31^3) no longer fit it: other kernels take those.
   const size_t fit = kTeamIcShared / 16 * 16 - 8 * (((size_t)n + 2) / 2);
   const int cap = packed ? (int)(std::min(std::min(kTeamIcRing, fit) & ~(size_t)15, blob.size()) / 16) : 0;
-  if (packed && ic_ring_places(desc, cap, kTeamIcBars)) {
-    for (size_t l = 0; l + 1 < desc.size(); ++l)  // each block names the next one's place
-      memcpy(blob.data() + (size_t)desc[l].from * 16 + 8, &desc[l + 1].at, 4);
+  packed = packed && ic_ring_places(desc, cap, kTeamIcBars);
+  if (packed) {
+    size_t b = 0;
+    for (const Levels* L : {&fwd, &bwd})
+      for (int l = 0; l < L->depth; ++l, ++b) {
+        unsigned char* o = blob.data() + (size_t)desc[b].from * 16;
+        const int ng = (L->start[l + 1] - L->start[l] + 31) / 32;
+        const size_t quads = quads_of[b], group = 256 + 768 * quads;
+        ((int*)o)[0] = ng;
+        ((int*)o)[1] = (int)quads;
+        ((int*)o)[2] = b + 1 < desc.size() ? desc[b + 1].at : 0;
+        ((int*)o)[3] = (int)group;
+        for (int g = 0; g < ng; ++g) {
+          unsigned char* og = o + 16 + g * group;
+          std::fill_n((unsigned short*)(og + 256), 128 * quads, (unsigned short)n);
+          for (int t = 0; t < 32; ++t) ((uint2*)og)[t] = make_uint2(0xffffu, 0u);
+        }
+      }
+    each_row([&](int i, int e0, int e1, uint2* meta, unsigned short* cols, float*) {
+      meta->x = (unsigned)i;
+      for (int e = e0; e < e1; ++e) cols[(e - e0) / 4 * 128 + (e - e0) % 4] = (unsigned short)hci[e];
+    });
+  }
+  unsigned bits = 0;
+  CK(ctx, cudaMemcpyAsync(&bits, err.p, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+  CK(ctx, cudaStreamSynchronize(s));
+  if (bits) {
+    M->ic_fail = bits;
+    return ic0_error(ctx, bits);
+  }
+  auto upload = [&](const Levels& L, DevBuf& out, DevBuf& starts, int& width, int& nlev) -> mpcg_status {
+    width = L.width;
+    nlev = L.depth;
+    CK(ctx, starts.ensure(4 * (size_t)(L.depth + 1)));
+    CK(ctx, cudaMemcpy(starts.p, L.start.data(), 4 * (size_t)(L.depth + 1), cudaMemcpyHostToDevice));
+    CK(ctx, out.ensure(4 * (size_t)std::max(n, 1)));
+    if (n) CK(ctx, cudaMemcpy(out.p, L.perm.data(), 4 * (size_t)n, cudaMemcpyHostToDevice));
+    return MPCG_OK;
+  };
+  mpcg_status ls = upload(fwd, M->icpf, M->icof, M->icwf, M->nlevf);
+  if (ls != MPCG_OK) return ls;
+  ls = upload(bwd, M->icpb, M->icob, M->icwb, M->nlevb);
+  if (ls != MPCG_OK) return ls;
+  if (packed) {
+    CK(ctx, cudaMemcpy(hF.data(), M->icf.p, 4 * (size_t)nnz, cudaMemcpyDeviceToHost));
+    each_row([&](int i, int e0, int e1, uint2* meta, unsigned short*, float* vals) {
+      memcpy(&meta->y, &hF[hdp[i]], 4);
+      for (int e = e0; e < e1; ++e) vals[(e - e0) / 4 * 128 + (e - e0) % 4] = hF[e];
+    });
     static_assert(sizeof(IcBlock) == sizeof(int4), "the kernel reads blocks as int4");
     if (M->icblob.ensure(blob.size()) != cudaSuccess ||
         M->icdesc.ensure(sizeof(IcBlock) * desc.size()) != cudaSuccess) {
